@@ -220,10 +220,8 @@ def measured_peaks():
 def kernel_bytes_per_node(nh: int) -> dict:
     f = 4
     return {
-        "k_moments": f * (9 * nh + nh),
-        "k_fields": f * (nh + 9 + 1 + 3 + 3 + 1 + 1),
-        "k_sources": f * (nh + nh + nh),
-        "k_collide": f * (9 + nh + 3 + 1 + 2 + 1 + nh + 9 + 9 * nh),
+        "k_fields_step": f * (9 * nh + 9 + 1 + nh + 3 + 3 + 1 + 1),
+        "k_collide_step": f * (9 + nh + 3 + 1 + 2 + 1 + nh + 9 + 9 * nh),
     }
 
 

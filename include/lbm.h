@@ -91,7 +91,7 @@ typedef struct {
                           follow f(t+1) = (f(t) + U f_(nx-2)(t+1)) / (1 + U), U the node's
                           x velocity clamped to [0, 1], then share the shift that sets the
                           node's pressure sum_a g_a to 0.  Needs nx >= 4, the population
-                          state (collapse_h 0, storage 0); runs on the multi-pass kernels;
+                          state (collapse_h 0, storage 0); runs on the two-kernel step;
                           not in batches. */
   double u_in;         /* inlet velocity (open_x) */
   double c_in[2];      /* inflow composition C_1, C_2 (open_x) */

@@ -544,7 +544,7 @@ lbm_status lbm_load(lbm_handle *h, const char *path) {
 int lbm_kernels_per_step(const lbm_handle *h) { return h ? h->kernels_per_step() : 0; }
 
 const char *lbm_kernel_name(const lbm_handle *h, int i) {
-  static const char *names[lbm::kSplitKernels] = {"k_moments", "k_fields", "k_sources", "k_collide"};
+  static const char *names[lbm::kSplitKernels] = {"k_fields_step", "k_collide_step"};
   if (!h || i < 0 || i >= h->kernels_per_step()) return "";
   if (!h->fused()) return names[i];
   lbm_handle *m = const_cast<lbm_handle *>(h);

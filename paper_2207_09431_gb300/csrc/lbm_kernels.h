@@ -29,8 +29,8 @@ struct StepBuffers {
 
 // Launches one step; if ev is non-null, records ev[i] before kernel i and
 // ev[nkernels] after the last one.
-constexpr int kSplitKernels = 4;
-void launch_split_step(const DevParams &P, const StepBuffers &B, cudaStream_t s, cudaEvent_t *ev = nullptr);
+constexpr int kSplitKernels = 2;
+cudaError_t launch_split_step(const DevParams &P, const StepBuffers &B, cudaStream_t s, cudaEvent_t *ev = nullptr);
 // Buffers of the fused single-kernel step.  shear and SV may be null (no
 // diagnostics written).
 struct FusedBuffers {

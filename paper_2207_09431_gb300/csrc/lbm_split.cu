@@ -1,14 +1,16 @@
-// Multi-pass form of the coupled D2Q9 step (arXiv 2207.09431, Sec. 2.2-2.3):
-//   k_moments  C_i = sum_a h_a^i                         (Eq. 22)
-//   k_fields   rho, mu (Eq. 5), u (Eq. 23), p (Eq. 24/R3), new tau (Eq. 25-33)
-//   k_sources  S_i + V_i = D_i lap(mu_i) + variable-mobility term (Eq. 6, 21)
-//   k_collide  collision of g (Eq. 14) and h (Eq. 18), pushed to the
-//              neighbours with half-way bounce-back and the destination-side
-//              source term (R9)
-// The intermediate fields live in scratch planes carved from the caller's
-// arena.  One thread per node; all arithmetic FP32.
+// Two-kernel form of the coupled D2Q9 step (arXiv 2207.09431, Sec. 2.2-2.3) for
+// the mixed difference scheme and the open x boundaries:
+//   k_fields_step   C_i = sum_a h_a^i (Eq. 22), rho, mu (Eq. 5), u (Eq. 23),
+//                   p (Eq. 24/R3), new tau (Eq. 25-33)
+//   k_collide_step  S_i + V_i (Eq. 6, 18, 21), collision of g (Eq. 14) and h (Eq.
+//                   18), streaming with half-way bounce-back or the open boundaries,
+//                   the destination-side source term (R9)
+// The fields between the two live in scratch planes carved from the caller's
+// arena.  All arithmetic FP32.  Also the macro fields, the initial equilibria and
+// the observables.
 #include "lbm_device.cuh"
 #include "lbm_kernels.h"
+#include "lbm_node.cuh"
 
 namespace lbm {
 
@@ -59,19 +61,27 @@ struct NodeCtx {
   float dC[3][9], drho[9], dp[9];
 };
 
-// Gathers C (radius 1 or 2), rho (from C), p (radius 1 or 2) around (x, y).
+// Field values around a node, from the planes.
+struct PlaneReader {
+  const DevParams &P;
+  CReader cr;
+  const float *pf;
+  int x, y;
+  __device__ __forceinline__ void C(int dx, int dy, float c[3]) const { cr.at(shifted(P, x, y, dx, dy), c); }
+  __device__ __forceinline__ float rho(int, int, const float c[3]) const { return rho_of(P, c[0], c[1], c[2]); }
+  __device__ __forceinline__ float p(int dx, int dy) const { return pf[shifted(P, x, y, dx, dy)]; }
+};
+
+// Gathers C (radius 1 or 2), rho (from C), p (radius 1 or 2) around a node.
 // Inlined, so that NodeCtx stays in registers.
-__device__ __forceinline__ void gather_gradients(const DevParams &P, const CReader &cr, const float *pf, int x, int y,
-                                 NodeCtx &n) {
-  const long long k0 = node_index(P, x, y);
+template <typename Reader>
+__device__ __forceinline__ void gather_gradients(int fd_scheme, const Reader &at, NodeCtx &n) {
   float Cn[9][3], rn[9], pn[9];
   for (int a = 0; a < 9; ++a) {
-    long long k = shifted(P, x, y, ex(a), ey(a));
-    cr.at(k, Cn[a]);
-    rn[a] = rho_of(P, Cn[a][0], Cn[a][1], Cn[a][2]);
-    pn[a] = pf[k];
+    at.C(ex(a), ey(a), Cn[a]);
+    rn[a] = at.rho(ex(a), ey(a), Cn[a]);
+    pn[a] = at.p(ex(a), ey(a));
   }
-  (void)k0;
   for (int j = 0; j < 3; ++j) {
     n.C[j] = Cn[0][j];
     float sx = 0.f, sy = 0.f;
@@ -100,15 +110,14 @@ __device__ __forceinline__ void gather_gradients(const DevParams &P, const CRead
   for (int a = 0; a < 9; ++a) {
     const int o = opp(a);
     float C2e[3] = {0.f, 0.f, 0.f}, r2e = 0.f, p2e = 0.f;
-    if (P.fd_scheme == 1) {
-      long long k2 = shifted(P, x, y, 2 * ex(a), 2 * ey(a));
-      cr.at(k2, C2e);
-      r2e = rho_of(P, C2e[0], C2e[1], C2e[2]);
-      p2e = pf[k2];
+    if (fd_scheme == 1) {
+      at.C(2 * ex(a), 2 * ey(a), C2e);
+      r2e = at.rho(2 * ex(a), 2 * ey(a), C2e);
+      p2e = at.p(2 * ex(a), 2 * ey(a));
     }
-    for (int j = 0; j < 3; ++j) n.dC[j][a] = dir_deriv(P.fd_scheme, Cn[o][j], Cn[0][j], Cn[a][j], C2e[j]);
-    n.drho[a] = dir_deriv(P.fd_scheme, rn[o], rn[0], rn[a], r2e);
-    n.dp[a] = dir_deriv(P.fd_scheme, pn[o], pn[0], pn[a], p2e);
+    for (int j = 0; j < 3; ++j) n.dC[j][a] = dir_deriv(fd_scheme, Cn[o][j], Cn[0][j], Cn[a][j], C2e[j]);
+    n.drho[a] = dir_deriv(fd_scheme, rn[o], rn[0], rn[a], r2e);
+    n.dp[a] = dir_deriv(fd_scheme, pn[o], pn[0], pn[a], p2e);
   }
 }
 
@@ -150,20 +159,13 @@ __global__ void k_moments(DevParams P, const float *__restrict__ h, float *__res
   }
 }
 
-// The fields of node (x, y) from the order parameters around it and its g
-// (Eq. 5, 22-24): C and rho at the node and its neighbours, grad C, lap C,
-// grad rho, mu_1..3, the forces, the moments of g and u.  Shared by k_fields
-// and the observables, so that both see the same velocity.
-template <int NH>
-__device__ __forceinline__ void fields_core(const DevParams &P, const float *__restrict__ Cf,
-                                            const float *__restrict__ g, int x, int y, long long k, NodeCtx &n,
-                                            float (&Cn)[9][3], float (&rn)[9], float (&ga)[9], float &m0) {
-  CReader cr{Cf, P.plane, NH};
-  for (int a = 0; a < 9; ++a) {
-    long long kk = shifted(P, x, y, ex(a), ey(a));
-    cr.at(kk, Cn[a]);
-    rn[a] = rho_of(P, Cn[a][0], Cn[a][1], Cn[a][2]);
-  }
+// The fields of a node from the order parameters around it and its g (Eq. 5,
+// 22-24): grad C, lap C, grad rho, mu_1..3, the forces, the moments of g and u,
+// from C and rho at the node and its neighbours.  Shared by every kernel that
+// computes fields and the observables, so that all see the same velocity.
+template <bool ROUND_FB>
+__device__ __forceinline__ void fields_math(const DevParams &P, NodeCtx &n, const float (&Cn)[9][3],
+                                            const float (&rn)[9], const float (&ga)[9], float &m0) {
   float lapC[3];
   for (int j = 0; j < 3; ++j) {
     n.C[j] = Cn[0][j];
@@ -191,11 +193,10 @@ __device__ __forceinline__ void fields_core(const DevParams &P, const float *__r
   n.Fs[0] = n.mu[0] * n.gC[0][0] + n.mu[1] * n.gC[1][0] + n.mu[2] * n.gC[2][0];
   n.Fs[1] = n.mu[0] * n.gC[0][1] + n.mu[1] * n.gC[1][1] + n.mu[2] * n.gC[2][1];
   n.Fb[0] = P.force_x;
-  n.Fb[1] = -n.rho * P.gravity;
+  n.Fb[1] = ROUND_FB ? __fmul_rn(-n.rho, P.gravity) : -n.rho * P.gravity;
   m0 = 0.f;
   float mx = 0.f, my = 0.f;
   for (int a = 0; a < 9; ++a) {
-    ga[a] = g[pop_index(k, a, 9)];
     m0 += ga[a];
     mx += ex(a) * ga[a];
     my += ey(a) * ga[a];
@@ -204,38 +205,146 @@ __device__ __forceinline__ void fields_core(const DevParams &P, const float *__r
   n.uy = (3.0f * my + 0.5f * (n.Fs[1] + n.Fb[1])) / n.rho;
 }
 
-// rho, mu_1..3, u, p and (if write_tau) the new relaxation time and strain rate.
+// fields_math of node (x, y) from the C planes.
+template <int NH, bool ROUND_FB>
+__device__ __forceinline__ void fields_core(const DevParams &P, const float *__restrict__ Cf,
+                                            const float *__restrict__ g, int x, int y, long long k, NodeCtx &n,
+                                            float (&Cn)[9][3], float (&rn)[9], float (&ga)[9], float &m0) {
+  CReader cr{Cf, P.plane, NH};
+  for (int a = 0; a < 9; ++a) {
+    long long kk = shifted(P, x, y, ex(a), ey(a));
+    cr.at(kk, Cn[a]);
+    rn[a] = rho_of(P, Cn[a][0], Cn[a][1], Cn[a][2]);
+  }
+  for (int a = 0; a < 9; ++a) ga[a] = g[pop_index(k, a, 9)];
+  fields_math<ROUND_FB>(P, n, Cn, rn, ga, m0);
+}
+
+// mu_1..3, u, p of the current state (for lbm_get_field).
 template <int NH>
-__global__ void k_fields(DevParams P, const float *__restrict__ Cf, const float *__restrict__ g,
-                         const float *__restrict__ tau_prev, float *__restrict__ mu, float *__restrict__ pf,
-                         float *__restrict__ uxf, float *__restrict__ uyf, float *__restrict__ tau_new,
-                         float *__restrict__ shear, unsigned *err, int write_tau) {
+__global__ void k_fields(DevParams P, const float *__restrict__ Cf, const float *__restrict__ g, float *__restrict__ mu,
+                         float *__restrict__ pf, float *__restrict__ uxf, float *__restrict__ uyf) {
   int x, y;
   if (!node_of_thread(P, x, y)) return;
   const long long k = node_index(P, x, y);
-  CReader cr{Cf, P.plane, NH};
   float Cn[9][3], rn[9], ga[9], m0;
   NodeCtx n;
-  fields_core<NH>(P, Cf, g, x, y, k, n, Cn, rn, ga, m0);
+  fields_core<NH, true>(P, Cf, g, x, y, k, n, Cn, rn, ga, m0);
+  for (int j = 0; j < 3; ++j) mu[(long long)j * P.plane + k] = n.mu[j];
+  pf[k] = m0 + 0.5f * kCs2 * (n.ux * n.grho[0] + n.uy * n.grho[1]);
+  uxf[k] = n.ux;
+  uyf[k] = n.uy;
+}
+
+// Row and column whose values stand at (x, y) of a tile and its rings: periodic, or
+// the mirror ghost rows beyond walls and ghost columns beyond the open ends
+// (slots far outside, of ragged tiles, hold some value that nothing reads).
+__device__ __forceinline__ long long tile_node(const DevParams &P, int x, int y) {
+  int xs;
+  if (!P.open_x) {
+    xs = wrap_periodic(x, P.nx);
+  } else {
+    xs = x < 0 ? -1 - x : (x >= P.nx ? 2 * P.nx - 1 - x : x);
+    xs = xs < 0 ? 0 : (xs >= P.nx ? P.nx - 1 : xs);
+  }
+  return node_index(P, xs, row_read(y, P.ny, P.periodic_y));
+}
+
+// Both step kernels take a tile of 32 x 4 output nodes per CTA and keep the
+// stencil neighbourhoods in shared memory: one load and one density per node and
+// ring slot, where a node's stencils of up to 25 points used to read the planes through
+// L1 and form rho again at every point.  The kernels were four (moments, fields, sources,
+// collision) and, with open ends, a fifth that walked the boundary rows: the
+// sources and the open ends are now part of the collision kernel, whose post-collision
+// populations of the tile and its one-node ring stay in shared memory and are
+// gathered by the node they arrive at (coalesced stores; the ring's collisions, a third
+// more, are computed twice).  Bound by the latency of two short kernels on small
+// lattices and by instruction issue on large ones.  Measured on a GB300, one step in
+// a replayed graph, two kernels against four (five): mixed scheme 64 x 128 11.0 against
+// 22.3 us, 200 x 400 18.0 against 29.6 us, 1024 x 2048 223 against 431 us; open channel
+// 240 x 60 11.0 against 31.2 us.  Tiles of 8 rows (fewer collisions twice, fewer CTAs)
+// ran 1 to 5 % slower above 400 x 800 at their best register budget and up to 10 % slower
+// on small lattices.  The order of a node's operations is that of the earlier kernels.
+constexpr int kTileX = 32, kTileY = 4;
+
+// Whether a tile at (x0, y0) and R nodes around it lie inside the lattice: then a
+// slot's node is at a fixed offset and nothing wraps or mirrors.
+__device__ __forceinline__ bool tile_inside(const DevParams &P, int x0, int y0, int r) {
+  return x0 >= r && y0 >= r && x0 + kTileX + r <= P.nx && y0 + kTileY + r <= P.ny;
+}
+
+// Shared-memory slots of a tile with a ring of R nodes.
+template <int R>
+struct Ring {
+  static constexpr int W = kTileX + 2 * R, H = kTileY + 2 * R, N = W * H;
+  static __device__ __forceinline__ int slot(int lx, int ly) { return (ly + R) * W + lx + R; }
+};
+
+// C_i, rho, mu_1..3, u, p, the new relaxation time and the strain rate.
+// SCHEME 1: directional derivatives reach two nodes.
+template <int NH, int SCHEME>
+__global__ void __launch_bounds__(kTileX *kTileY)
+    k_fields_step(DevParams P, const float *__restrict__ h, const float *__restrict__ g,
+                  const float *__restrict__ tau_prev, float *__restrict__ Cf, float *__restrict__ mu,
+                  float *__restrict__ pf, float *__restrict__ uxf, float *__restrict__ uyf,
+                  float *__restrict__ tau_new, float *__restrict__ shear, unsigned *err) {
+  using S = Ring<1 + SCHEME>;
+  __shared__ float sC[NH][S::N], srho[S::N];
+  const int t = threadIdx.x, x0 = blockIdx.x * kTileX, y0 = blockIdx.y * kTileY;
+  const int tx = t % kTileX, ty = t / kTileX, x = x0 + tx, y = y0 + ty;
+  const bool mine = x < P.nx && y < P.ny;
+  const long long k = node_index(P, x, y);
+  float ga[9], tp = 0.f;
+  if (mine) {
+#pragma unroll
+    for (int a = 0; a < 9; ++a) ga[a] = g[pop_index(k, a, 9)];
+    tp = tau_prev[k];
+  }
+  const bool inside = tile_inside(P, x0, y0, 1 + SCHEME);
+  for (int q = t; q < S::N; q += kTileX * kTileY) {
+    const int xq = x0 + q % S::W - (1 + SCHEME), yq = y0 + q / S::W - (1 + SCHEME);
+    const long long kq = inside ? node_index(P, xq, yq) : tile_node(P, xq, yq);
+    float c[2] = {0.f, 0.f};
+#pragma unroll
+    for (int i = 0; i < NH; ++i) {
+      float s = 0.f;
+#pragma unroll
+      for (int a = 0; a < 9; ++a) s += h[pop_index(kq, i * 9 + a, 9 * NH)];
+      sC[i][q] = c[i] = s;
+    }
+    srho[q] = rho_of(P, c[0], c[1], 1.0f - c[0] - c[1]);
+  }
+  __syncthreads();
+  if (!mine) return;
+  auto read = [&](int dx, int dy, float c[3]) {
+    const int q = S::slot(tx + dx, ty + dy);
+    c[0] = sC[0][q];
+    c[1] = NH == 2 ? sC[NH - 1][q] : 0.0f;
+    c[2] = 1.0f - c[0] - c[1];
+    return srho[q];
+  };
+  NodeCtx n;
+  float Cn[9][3], rn[9], m0;
+#pragma unroll
+  for (int a = 0; a < 9; ++a) rn[a] = read(ex(a), ey(a), Cn[a]);
+  fields_math<true>(P, n, Cn, rn, ga, m0);
   n.p = m0 + 0.5f * kCs2 * (n.ux * n.grho[0] + n.uy * n.grho[1]);
+#pragma unroll
+  for (int i = 0; i < NH; ++i) Cf[(long long)i * P.plane + k] = n.C[i];
+#pragma unroll
   for (int j = 0; j < 3; ++j) mu[(long long)j * P.plane + k] = n.mu[j];
   pf[k] = n.p;
   uxf[k] = n.ux;
   uyf[k] = n.uy;
-  if (!write_tau) return;
   // directional derivatives of rho and C (the g forcing has no p derivative)
   for (int a = 0; a < 9; ++a) {
     const int o = opp(a);
     float C2e[3] = {0.f, 0.f, 0.f}, r2e = 0.f;
-    if (P.fd_scheme == 1) {
-      cr.at(shifted(P, x, y, 2 * ex(a), 2 * ey(a)), C2e);
-      r2e = rho_of(P, C2e[0], C2e[1], C2e[2]);
-    }
-    for (int j = 0; j < 3; ++j) n.dC[j][a] = dir_deriv(P.fd_scheme, Cn[o][j], Cn[0][j], Cn[a][j], C2e[j]);
-    n.drho[a] = dir_deriv(P.fd_scheme, rn[o], rn[0], rn[a], r2e);
+    if (SCHEME == 1) r2e = read(2 * ex(a), 2 * ey(a), C2e);
+    for (int j = 0; j < 3; ++j) n.dC[j][a] = dir_deriv(SCHEME, Cn[o][j], Cn[0][j], Cn[a][j], C2e[j]);
+    n.drho[a] = dir_deriv(SCHEME, rn[o], rn[0], rn[a], r2e);
   }
   // strain rate from the non-equilibrium part with the previous tau (R23)
-  const float tp = tau_prev[k];
   const float fac = 3.0f * (2.0f * tp / (2.0f * tp + 1.0f));
   float Pxx = 0.f, Pyy = 0.f, Pxy = 0.f;
   for (int a = 0; a < 9; ++a) {
@@ -256,169 +365,217 @@ __global__ void k_fields(DevParams P, const float *__restrict__ Cf, const float 
   if (!(isfinite(n.rho) && isfinite(n.p) && isfinite(n.ux) && isfinite(n.uy) && isfinite(tn))) atomicOr(err, 1u);
 }
 
-// S_i + V_i (Eq. 6, 18, 21; R8) for every transported order parameter.
-__global__ void k_sources(DevParams P, const float *__restrict__ Cf, const float *__restrict__ mu,
-                          float *__restrict__ SV) {
-  int x, y;
-  if (!node_of_thread(P, x, y)) return;
-  const long long k = node_index(P, x, y);
-  for (int i = 0; i < P.nh; ++i) {
-    const float *Ci = Cf + (long long)i * P.plane;
-    const float *mi = mu + (long long)i * P.plane;
-    float gcx = 0.f, gcy = 0.f, gmx = 0.f, gmy = 0.f, lm = 0.f;
-    const float m0 = mi[k];
-    for (int a = 0; a < 9; ++a) {
-      long long kk = shifted(P, x, y, ex(a), ey(a));
-      float cv = Ci[kk], mv = mi[kk];
-      gcx += wt(a) * ex(a) * cv;
-      gcy += wt(a) * ey(a) * cv;
-      gmx += wt(a) * ex(a) * mv;
-      gmy += wt(a) * ey(a) * mv;
-      lm += wt(a) * (mv - m0);
-    }
-    const float lapmu = 6.0f * lm;
-    const float C = Ci[k];
-    const float D0s = P.d0_sig[i];
-    float s;
-    if (P.mobility == 1) {
-      // mobility with C clipped to [0, 1] and its derivative (reading R8)
-      const float cc = fminf(fmaxf(C, 0.0f), 1.0f);
-      const float dv = (C >= 0.0f && C <= 1.0f)
-                           ? D0s * (1.0f - 2.0f * C) * (3.0f * gcx * 3.0f * gmx + 3.0f * gcy * 3.0f * gmy)
-                           : 0.0f;
-      s = D0s * cc * (1.0f - cc) * lapmu + dv;
-    } else {
-      s = D0s * lapmu;
-    }
-    SV[(long long)i * P.plane + k] = s;
-  }
-}
-
-// Collision of g (Eq. 14) and h (Eq. 18, tau_h = 1/2) at each node, pushed to
-// x + e_a; populations that would cross a wall return to x in the opposite
-// direction.  With tau_h = 1/2 the BGK step of Eq. 18 replaces h by its
-// modified equilibrium, so h itself is not read: h* = C Gamma + Phi/2 + SV Gamma/2.
-template <int NH>
-__global__ void k_collide(DevParams P, const float *__restrict__ g, const float *__restrict__ Cf,
-                          const float *__restrict__ mu, const float *__restrict__ pf, const float *__restrict__ uxf,
-                          const float *__restrict__ uyf, const float *__restrict__ tau_new,
-                          const float *__restrict__ SV, float *__restrict__ g_out, float *__restrict__ h_out) {
-  int x, y;
-  if (!node_of_thread(P, x, y)) return;
-  const long long k = node_index(P, x, y);
-  CReader cr{Cf, P.plane, NH};
-  NodeCtx n;
-  gather_gradients(P, cr, pf, x, y, n);
-  n.ux = uxf[k];
-  n.uy = uyf[k];
-  for (int j = 0; j < 3; ++j) n.mu[j] = mu[(long long)j * P.plane + k];
-  n.Fs[0] = n.mu[0] * n.gC[0][0] + n.mu[1] * n.gC[1][0] + n.mu[2] * n.gC[2][0];
-  n.Fs[1] = n.mu[0] * n.gC[0][1] + n.mu[1] * n.gC[1][1] + n.mu[2] * n.gC[2][1];
-  n.Fb[0] = P.force_x;
-  n.Fb[1] = -n.rho * P.gravity;
-  const float omega = 1.0f / (tau_new[k] + 0.5f);
-  float sv[2] = {0.f, 0.f};
-#pragma unroll
-  for (int i = 0; i < 2; ++i)
-    if (i < NH) sv[i] = SV[(long long)i * P.plane + k];
-#pragma unroll
+// S_i + V_i (Eq. 6, 18, 21; R8) from the stencils of C_i and mu_i around a node.
+__device__ __forceinline__ float source_of(const DevParams &P, int i, const float (&cv)[9], const float (&mv)[9]) {
+  float gcx = 0.f, gcy = 0.f, gmx = 0.f, gmy = 0.f, lm = 0.f;
   for (int a = 0; a < 9; ++a) {
-    const float G = gamma_a(a, n.ux, n.uy);
-    const float pg = phi_g(n, a, G);
-    const float geq = wt(a) * n.p + n.rho * kCs2 * (G - wt(a)) - 0.5f * pg;
-    const float gv = g[pop_index(k, a, 9)];
-    const float gstar = gv - omega * (gv - geq) + pg;
-    // destination
-    int dx = x + ex(a), dy = y + ey(a);
-    int da = a;
-    long long kd;
-    if (!P.periodic_y && (dy < 0 || dy >= P.ny)) {
-      kd = k;
-      da = opp(a);
-    } else if (P.open_x && (dx < 0 || dx >= P.nx)) {
-      continue;  // leaves through the inlet or outlet; k_open_x sets what enters
-    } else {
-      kd = node_index(P, wrap_x(dx, P.nx), P.periodic_y ? wrap_y(dy, P.ny, 1) : dy);
-    }
-    g_out[pop_index(kd, da, 9)] = gstar;
-    const float Gd = gamma_a(da, uxf[kd], uyf[kd]);
-#pragma unroll
-    for (int i = 0; i < 2; ++i) {
-      if (i >= NH) break;
-      const float ph = phi_h(n, i, a, G);
-      const float hstar = n.C[i] * G + 0.5f * ph + 0.5f * sv[i] * G;
-      h_out[pop_index(kd, i * 9 + da, 9 * NH)] = hstar + 0.5f * SV[(long long)i * P.plane + kd] * Gd;
-    }
+    gcx += wt(a) * ex(a) * cv[a];
+    gcy += wt(a) * ey(a) * cv[a];
+    gmx += wt(a) * ex(a) * mv[a];
+    gmy += wt(a) * ey(a) * mv[a];
+    lm += wt(a) * (mv[a] - mv[0]);
   }
+  const float lapmu = 6.0f * lm;
+  const float C = cv[0];
+  const float D0s = P.d0_sig[i];
+  if (P.mobility == 1) {
+    // mobility with C clipped to [0, 1] and its derivative (reading R8)
+    const float cc = fminf(fmaxf(C, 0.0f), 1.0f);
+    const float dv = (C >= 0.0f && C <= 1.0f)
+                         ? D0s * (1.0f - 2.0f * C) * (3.0f * gcx * 3.0f * gmx + 3.0f * gcy * 3.0f * gmy)
+                         : 0.0f;
+    return D0s * cc * (1.0f - cc) * lapmu + dv;
+  }
+  return D0s * lapmu;
 }
 
-// Populations entering through the open x boundaries, after k_collide (one
-// thread per row).  Inlet (x = 0, e_x = +1): g from a ghost column x = -1 whose
-// post-collision g is the equilibrium w p + rho cs^2 (Gamma - w) at (u_in, 0)
-// plus the non-equilibrium part of column 0's post-collision g (which k_collide
-// stored at column 1), h the equilibrium c_in Gamma(u_in) plus the node's
-// destination-side term.  Outlet (x = nx - 1, e_x = -1): the convective
-// condition f(t+1) = (f(t) + U f_(nx-2)(t+1)) / (1 + U), U the node's x velocity
-// clamped to [0, 1], then the shift (shared by weight among the entering g)
-// that sets the node's pressure sum_a g_a to 0.  Wall rows keep bounce-back.
-__global__ void k_open_x(DevParams P, const float *__restrict__ g_old, const float *__restrict__ h_old,
-                         const float *__restrict__ Cf, const float *__restrict__ pf, const float *__restrict__ uxf,
-                         const float *__restrict__ uyf, const float *__restrict__ SV, float *__restrict__ g_out,
-                         float *__restrict__ h_out) {
-  const int y = blockIdx.x * blockDim.x + threadIdx.x;
-  if (y >= P.ny) return;
-  const long long pl = P.plane;
-  CReader cr{Cf, P.plane, P.nh};
-  // inlet
-  {
-    const long long k = node_index(P, 0, y), k1 = node_index(P, 1, y);
-    for (int a = 0; a < 9; ++a) {
-      if (ex(a) != 1) continue;
-      int sy = y - ey(a);
-      if (!P.periodic_y && (sy < 0 || sy >= P.ny)) continue;
-      sy = wrap_y(sy, P.ny, P.periodic_y);
-      const long long k0 = node_index(P, 0, sy);
-      float c[3];
-      cr.at(k0, c);
-      const float rho = rho_of(P, c[0], c[1], c[2]);
-      const float p = pf[k0];
-      const float w = wt(a);
-      const float eq_in = w * p + rho * kCs2 * (gamma_a(a, P.u_in, 0.0f) - w);
-      const float eq_0 = w * p + rho * kCs2 * (gamma_a(a, uxf[k0], uyf[k0]) - w);
-      g_out[pop_index(k, a, 9)] = eq_in + (g_out[pop_index(k1, a, 9)] - eq_0);
-      const float G = gamma_a(a, uxf[k], uyf[k]);
-      const float Gin = gamma_a(a, P.u_in, 0.0f);
-      for (int i = 0; i < P.nh; ++i)
-        h_out[pop_index(k, i * 9 + a, 9 * P.nh)] = P.c_in[i] * Gin + 0.5f * SV[(long long)i * pl + k] * G;
+template <int NH, int SCHEME>
+struct CollideSmem {
+  using RC = Ring<2 + SCHEME>;
+  using RM = Ring<2>;
+  using R1 = Ring<1>;
+  float C[NH][RC::N], rho[RC::N], p[RC::N], mu[NH][RM::N];
+  float g[9][R1::N], h[NH][9][R1::N], sv[NH][R1::N], ux[R1::N], uy[R1::N];
+};
+// Threads: the collisions of the tile and its ring in one pass.
+constexpr int kCollideThreads = (Ring<1>::N + 31) / 32 * 32;
+
+// Sources, collision and streaming of a tile.  With tau_h = 1/2 the BGK step of
+// Eq. 18 replaces h by its modified equilibrium, so h itself is read at the outlet only:
+// h* = C Gamma + Phi/2 + SV Gamma/2.  Populations that would cross a wall return in
+// the opposite direction.  Open x: at the inlet (x = 0, e_x = +1) g comes from a ghost
+// column x = -1 whose post-collision g is the equilibrium w p + rho cs^2 (Gamma - w) at
+// (u_in, 0) plus the non-equilibrium part of column 0's post-collision g, h the
+// equilibrium c_in Gamma(u_in) plus the node's destination-side term; at the outlet
+// (x = nx - 1, e_x = -1) the convective condition f(t+1) = (f(t) + U f_(nx-2)(t+1)) / (1 + U),
+// U the node's x velocity clamped to [0, 1], then the shift (shared by weight among
+// the entering g) that sets the node's pressure sum_a g_a to 0.  Wall rows keep bounce-back.
+template <int NH, int SCHEME, int MINB>
+__global__ void __launch_bounds__(kCollideThreads, MINB)
+    k_collide_step(DevParams P, const float *__restrict__ g, const float *__restrict__ h_old,
+                   const float *__restrict__ Cf, const float *__restrict__ mu, const float *__restrict__ pf,
+                   const float *__restrict__ uxf, const float *__restrict__ uyf, const float *__restrict__ tau_new,
+                   float *__restrict__ SV, float *__restrict__ g_out, float *__restrict__ h_out) {
+  using S = CollideSmem<NH, SCHEME>;
+  using RC = typename S::RC;
+  using RM = typename S::RM;
+  using R1 = typename S::R1;
+  constexpr int NT = kCollideThreads;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  S &s = *reinterpret_cast<S *>(smem_raw);
+  const int t = threadIdx.x, x0 = blockIdx.x * kTileX, y0 = blockIdx.y * kTileY;
+
+  // this thread's node of the one-node ring (real rows, and columns of the lattice)
+  const int lx = t % R1::W - 1, ly = t / R1::W - 1, xr = x0 + lx, yr = y0 + ly;
+  const bool ring = t < R1::N && (P.periodic_y || (yr >= 0 && yr < P.ny)) && (!P.open_x || (xr >= 0 && xr < P.nx));
+  const bool inside = tile_inside(P, x0, y0, 2 + SCHEME);
+  const long long kr = inside ? node_index(P, xr, yr) : tile_node(P, xr, yr);
+  NodeCtx n;
+  float gv[9], tn = 0.f;
+  if (ring) {
+#pragma unroll
+    for (int a = 0; a < 9; ++a) gv[a] = g[pop_index(kr, a, 9)];
+    tn = tau_new[kr];
+    n.ux = uxf[kr];
+    n.uy = uyf[kr];
+#pragma unroll
+    for (int j = 0; j < 3; ++j) n.mu[j] = mu[(long long)j * P.plane + kr];
+  }
+  for (int q = t; q < RC::N; q += NT) {
+    const int cx = q % RC::W - (2 + SCHEME), cy = q / RC::W - (2 + SCHEME);
+    const long long kq = inside ? node_index(P, x0 + cx, y0 + cy) : tile_node(P, x0 + cx, y0 + cy);
+    const float c0 = Cf[kq], c1 = NH == 2 ? Cf[P.plane + kq] : 0.0f;
+    s.C[0][q] = c0;
+    if (NH == 2) s.C[NH - 1][q] = c1;
+    s.rho[q] = rho_of(P, c0, c1, 1.0f - c0 - c1);
+    s.p[q] = pf[kq];
+    if (SCHEME == 0 || (cx >= -2 && cx < kTileX + 2 && cy >= -2 && cy < kTileY + 2)) {
+#pragma unroll
+      for (int i = 0; i < NH; ++i) s.mu[i][RM::slot(cx, cy)] = mu[(long long)i * P.plane + kq];
     }
   }
-  // outlet
-  {
-    const long long k = node_index(P, P.nx - 1, y), kin = node_index(P, P.nx - 2, y);
-    const float U = fminf(fmaxf(uxf[k], 0.0f), 1.0f);
-    const float inv = 1.0f / (1.0f + U);
-    float wsum = 0.f;
-    bool set[9];
+  __syncthreads();
+
+  if (ring) {
+    struct {
+      const S &s;
+      int lx, ly;
+      __device__ __forceinline__ int q(int dx, int dy) const { return RC::slot(lx + dx, ly + dy); }
+      __device__ __forceinline__ void C(int dx, int dy, float c[3]) const {
+        c[0] = s.C[0][q(dx, dy)];
+        c[1] = NH == 2 ? s.C[NH - 1][q(dx, dy)] : 0.0f;
+        c[2] = 1.0f - c[0] - c[1];
+      }
+      __device__ __forceinline__ float rho(int dx, int dy, const float *) const { return s.rho[q(dx, dy)]; }
+      __device__ __forceinline__ float p(int dx, int dy) const { return s.p[q(dx, dy)]; }
+    } at{s, lx, ly};
+    float sv[NH];
+#pragma unroll
+    for (int i = 0; i < NH; ++i) {
+      float cv[9], mv[9];
+#pragma unroll
+      for (int a = 0; a < 9; ++a) {
+        cv[a] = s.C[i][RC::slot(lx + ex(a), ly + ey(a))];
+        mv[a] = s.mu[i][RM::slot(lx + ex(a), ly + ey(a))];
+      }
+      sv[i] = source_of(P, i, cv, mv);
+      s.sv[i][t] = sv[i];
+    }
+    s.ux[t] = n.ux;
+    s.uy[t] = n.uy;
+    gather_gradients(SCHEME, at, n);
+    n.Fs[0] = n.mu[0] * n.gC[0][0] + n.mu[1] * n.gC[1][0] + n.mu[2] * n.gC[2][0];
+    n.Fs[1] = n.mu[0] * n.gC[0][1] + n.mu[1] * n.gC[1][1] + n.mu[2] * n.gC[2][1];
+    n.Fb[0] = P.force_x;
+    n.Fb[1] = -n.rho * P.gravity;
+    const float omega = 1.0f / (tn + 0.5f);
+#pragma unroll
     for (int a = 0; a < 9; ++a) {
-      set[a] = false;
-      if (ex(a) != -1) continue;
-      const int sy = y - ey(a);
-      if (!P.periodic_y && (sy < 0 || sy >= P.ny)) continue;
-      set[a] = true;
-      wsum += wt(a);
-      g_out[pop_index(k, a, 9)] = (g_old[pop_index(k, a, 9)] + U * g_out[pop_index(kin, a, 9)]) * inv;
-      for (int i = 0; i < P.nh; ++i) {
-        const int q = i * 9 + a, nq = 9 * P.nh;
-        h_out[pop_index(k, q, nq)] = (h_old[pop_index(k, q, nq)] + U * h_out[pop_index(kin, q, nq)]) * inv;
+      const float G = gamma_a(a, n.ux, n.uy);
+      // (which product of the equilibrium is rounded on its own is spelled out: left to the
+      // compiler it changes with the code around it, and the results by rounding)
+      const float pg = phi_g(n, a, G), Gw = G - wt(a), rc = n.rho * kCs2;
+      const float lin = a < 5 ? __fmaf_rn(wt(a), n.p, __fmul_rn(rc, Gw)) : __fmaf_rn(rc, Gw, __fmul_rn(wt(a), n.p));
+      const float geq = lin - 0.5f * pg;
+      s.g[a][t] = gv[a] - omega * (gv[a] - geq) + pg;
+#pragma unroll
+      for (int i = 0; i < NH; ++i) {
+        const float ph = phi_h(n, i, a, G);
+        s.h[i][a][t] = n.C[i] * G + 0.5f * ph + 0.5f * sv[i] * G;
       }
     }
-    if (wsum > 0.f) {
-      float p0 = 0.f;
-      for (int a = 0; a < 9; ++a) p0 += g_out[pop_index(k, a, 9)];
-      for (int a = 0; a < 9; ++a)
-        if (set[a]) g_out[pop_index(k, a, 9)] -= p0 * wt(a) / wsum;
+  }
+  __syncthreads();
+
+  // streaming: the populations that arrive at output node (x, y)
+  const int tx = t % kTileX, ty = t / kTileX, x = x0 + tx, y = y0 + ty;
+  if (ty >= kTileY || x >= P.nx || y >= P.ny) return;
+  const long long k = node_index(P, x, y);
+  const int q0 = R1::slot(tx, ty);
+  const float ux = s.ux[q0], uy = s.uy[q0];
+  float gy[9];
+  unsigned entered = 0;  // outlet: directions that enter there
+  float wsum = 0.f, U = 0.f, inv = 1.f;
+  const bool outlet = P.open_x && x == P.nx - 1;
+  if (outlet) {
+    U = fminf(fmaxf(ux, 0.0f), 1.0f);
+    inv = 1.0f / (1.0f + U);
+  }
+#pragma unroll
+  for (int i = 0; i < NH; ++i) SV[(long long)i * P.plane + k] = s.sv[i][q0];
+#pragma unroll
+  for (int a = 0; a < 9; ++a) {
+    const int sx = x - ex(a), sy = y - ey(a);
+    const float G = gamma_a(a, ux, uy);
+    if (!P.periodic_y && (sy < 0 || sy >= P.ny)) {  // returned by the wall
+      gy[a] = s.g[opp(a)][q0];
+#pragma unroll
+      for (int i = 0; i < NH; ++i)
+        h_out[pop_index(k, i * 9 + a, 9 * NH)] = s.h[i][opp(a)][q0] + 0.5f * s.sv[i][q0] * G;
+    } else if (P.open_x && sx < 0) {
+      const int q = R1::slot(tx, ty - ey(a));  // column 0 of the source row
+      const int qc = RC::slot(tx, ty - ey(a));
+      const float rho = s.rho[qc], p = s.p[qc], w = wt(a);
+      const float Gin = gamma_a(a, P.u_in, 0.0f);
+      const float rc = rho * kCs2, u0 = s.ux[q], v0 = s.uy[q];
+      const float eu = ex(a) * u0 + ey(a) * v0, uu = u0 * u0 + v0 * v0;
+      const float eq_in = __fmaf_rn(w, p, __fmul_rn(rc, __fsub_rn(Gin, w)));
+      const float eq_0 = __fmaf_rn(w, p, __fmul_rn(rc, __fmaf_rn(w, 1.0f + 3.0f * eu + 4.5f * eu * eu - 1.5f * uu, -w)));
+      gy[a] = eq_in + (s.g[a][q] - eq_0);
+#pragma unroll
+      for (int i = 0; i < NH; ++i)
+        h_out[pop_index(k, i * 9 + a, 9 * NH)] = P.c_in[i] * Gin + 0.5f * s.sv[i][q0] * G;
+    } else if (P.open_x && sx >= P.nx) {
+      const int q = R1::slot(tx, ty - ey(a));       // column nx - 1 of the source row
+      const int qi = R1::slot(tx - 1, ty);          // (nx - 2, y), where its population arrives
+      entered |= 1u << a;
+      wsum += wt(a);
+      gy[a] = (g[pop_index(k, a, 9)] + U * s.g[a][q]) * inv;
+      const float Gi = gamma_a(a, s.ux[qi], s.uy[qi]);
+#pragma unroll
+      for (int i = 0; i < NH; ++i) {
+        const float arrives = s.h[i][a][q] + 0.5f * s.sv[i][qi] * Gi;
+        const long long o = pop_index(k, i * 9 + a, 9 * NH);
+        h_out[o] = (h_old[o] + U * arrives) * inv;
+      }
+    } else {
+      const int q = R1::slot(tx - ex(a), ty - ey(a));
+      gy[a] = s.g[a][q];
+#pragma unroll
+      for (int i = 0; i < NH; ++i)
+        h_out[pop_index(k, i * 9 + a, 9 * NH)] = s.h[i][a][q] + 0.5f * s.sv[i][q0] * G;
     }
   }
+  if (outlet && wsum > 0.f) {
+    float p0 = 0.f;
+#pragma unroll
+    for (int a = 0; a < 9; ++a) p0 += gy[a];
+#pragma unroll
+    for (int a = 0; a < 9; ++a)
+      if (entered >> a & 1u) gy[a] -= p0 * wt(a) / wsum;
+  }
+#pragma unroll
+  for (int a = 0; a < 9; ++a) g_out[pop_index(k, a, 9)] = gy[a];
 }
 
 // Modified equilibria (Eq. 16, 20) of given C, p, u, and tau at zero strain
@@ -432,7 +589,7 @@ __global__ void k_init(DevParams P, const float *__restrict__ Cf, const float *_
   const long long k = node_index(P, x, y);
   CReader cr{Cf, P.plane, NH};
   NodeCtx n;
-  gather_gradients(P, cr, pf, x, y, n);
+  gather_gradients(P.fd_scheme, PlaneReader{P, cr, pf, x, y}, n);
   float Cn[9][3], lapC[3];
   for (int a = 0; a < 9; ++a) cr.at(shifted(P, x, y, ex(a), ey(a)), Cn[a]);
   for (int j = 0; j < 3; ++j) {
@@ -530,7 +687,7 @@ __global__ void __launch_bounds__(kObsThreads) k_obs_direct(DevParams P, const f
       const long long k = node_index(P, x, y);
       NodeCtx n;
       float Cn[9][3], rn[9], ga[9], m0;
-      fields_core<NH>(P, Cf, g, x, y, k, n, Cn, rn, ga, m0);
+      fields_core<NH, false>(P, Cf, g, x, y, k, n, Cn, rn, ga, m0);
       for (int i = 0; i < 3; ++i) {
         r[i].add(n.C[i]);
         r[3 + i].add(n.C[i] > 0.5f ? n.C[i] : 0.0f);
@@ -580,26 +737,24 @@ static dim3 node_grid(const DevParams &P, dim3 blk) {
   return dim3((P.nx + blk.x - 1) / blk.x, (P.ny + blk.y - 1) / blk.y);
 }
 
-void launch_split_step(const DevParams &P, const StepBuffers &B, cudaStream_t s, cudaEvent_t *ev) {
-  const dim3 blk(32, 8);
-  const dim3 grd = node_grid(P, blk);
+template <int NH, int SCHEME, int MINB>
+static cudaError_t split_step(const DevParams &P, const StepBuffers &B, cudaStream_t s, cudaEvent_t *ev) {
+  using S = CollideSmem<NH, SCHEME>;
+  static_assert(sizeof(S) <= 48 * 1024, "no opt-in for more shared memory");
+  const dim3 grd((P.nx + kTileX - 1) / kTileX, (P.ny + kTileY - 1) / kTileY);
   if (ev) cudaEventRecord(ev[0], s);
-  k_moments<<<grd, blk, 0, s>>>(P, B.h_in, B.C);
+  k_fields_step<NH, SCHEME><<<grd, kTileX * kTileY, 0, s>>>(P, B.h_in, B.g_in, B.tau_in, B.C, B.mu, B.p, B.ux, B.uy,
+                                                           B.tau_out, B.shear, B.err);
   if (ev) cudaEventRecord(ev[1], s);
-  if (P.nh == 1)
-    k_fields<1><<<grd, blk, 0, s>>>(P, B.C, B.g_in, B.tau_in, B.mu, B.p, B.ux, B.uy, B.tau_out, B.shear, B.err, 1);
-  else
-    k_fields<2><<<grd, blk, 0, s>>>(P, B.C, B.g_in, B.tau_in, B.mu, B.p, B.ux, B.uy, B.tau_out, B.shear, B.err, 1);
+  k_collide_step<NH, SCHEME, MINB><<<grd, kCollideThreads, sizeof(S), s>>>(
+      P, B.g_in, B.h_in, B.C, B.mu, B.p, B.ux, B.uy, B.tau_out, B.SV, B.g_out, B.h_out);
   if (ev) cudaEventRecord(ev[2], s);
-  k_sources<<<grd, blk, 0, s>>>(P, B.C, B.mu, B.SV);
-  if (ev) cudaEventRecord(ev[3], s);
-  if (P.nh == 1)
-    k_collide<1><<<grd, blk, 0, s>>>(P, B.g_in, B.C, B.mu, B.p, B.ux, B.uy, B.tau_out, B.SV, B.g_out, B.h_out);
-  else
-    k_collide<2><<<grd, blk, 0, s>>>(P, B.g_in, B.C, B.mu, B.p, B.ux, B.uy, B.tau_out, B.SV, B.g_out, B.h_out);
-  if (P.open_x)
-    k_open_x<<<(P.ny + 127) / 128, 128, 0, s>>>(P, B.g_in, B.h_in, B.C, B.p, B.ux, B.uy, B.SV, B.g_out, B.h_out);
-  if (ev) cudaEventRecord(ev[4], s);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_split_step(const DevParams &P, const StepBuffers &B, cudaStream_t s, cudaEvent_t *ev) {
+  if (P.nh == 1) return P.fd_scheme == 1 ? split_step<1, 1, 4>(P, B, s, ev) : split_step<1, 0, 4>(P, B, s, ev);
+  return P.fd_scheme == 1 ? split_step<2, 1, 2>(P, B, s, ev) : split_step<2, 0, 2>(P, B, s, ev);
 }
 
 void launch_macros(const DevParams &P, const StepBuffers &B, cudaStream_t s) {
@@ -607,9 +762,9 @@ void launch_macros(const DevParams &P, const StepBuffers &B, cudaStream_t s) {
   const dim3 grd = node_grid(P, blk);
   if (B.h_in) k_moments<<<grd, blk, 0, s>>>(P, B.h_in, B.C);  // null: the state holds C
   if (P.nh == 1)
-    k_fields<1><<<grd, blk, 0, s>>>(P, B.C, B.g_in, B.tau_in, B.mu, B.p, B.ux, B.uy, nullptr, nullptr, B.err, 0);
+    k_fields<1><<<grd, blk, 0, s>>>(P, B.C, B.g_in, B.mu, B.p, B.ux, B.uy);
   else
-    k_fields<2><<<grd, blk, 0, s>>>(P, B.C, B.g_in, B.tau_in, B.mu, B.p, B.ux, B.uy, nullptr, nullptr, B.err, 0);
+    k_fields<2><<<grd, blk, 0, s>>>(P, B.C, B.g_in, B.mu, B.p, B.ux, B.uy);
 }
 
 // Rows [y0, y1) of nplanes dense FP64 planes into the pitched FP32 planes.
