@@ -77,14 +77,17 @@ struct PlaneReader {
 template <typename Reader>
 __device__ __forceinline__ void gather_gradients(int fd_scheme, const Reader &at, NodeCtx &n) {
   float Cn[9][3], rn[9], pn[9];
+#pragma unroll
   for (int a = 0; a < 9; ++a) {
     at.C(ex(a), ey(a), Cn[a]);
     rn[a] = at.rho(ex(a), ey(a), Cn[a]);
     pn[a] = at.p(ex(a), ey(a));
   }
+#pragma unroll
   for (int j = 0; j < 3; ++j) {
     n.C[j] = Cn[0][j];
     float sx = 0.f, sy = 0.f;
+#pragma unroll
     for (int a = 0; a < 9; ++a) {
       sx += wt(a) * ex(a) * Cn[a][j];
       sy += wt(a) * ey(a) * Cn[a][j];
@@ -96,6 +99,7 @@ __device__ __forceinline__ void gather_gradients(int fd_scheme, const Reader &at
   n.p = pn[0];
   {
     float sx = 0.f, sy = 0.f, qx = 0.f, qy = 0.f;
+#pragma unroll
     for (int a = 0; a < 9; ++a) {
       sx += wt(a) * ex(a) * rn[a];
       sy += wt(a) * ey(a) * rn[a];
@@ -107,6 +111,7 @@ __device__ __forceinline__ void gather_gradients(int fd_scheme, const Reader &at
     n.gp[0] = 3.0f * qx;
     n.gp[1] = 3.0f * qy;
   }
+#pragma unroll
   for (int a = 0; a < 9; ++a) {
     const int o = opp(a);
     float C2e[3] = {0.f, 0.f, 0.f}, r2e = 0.f, p2e = 0.f;
@@ -115,6 +120,7 @@ __device__ __forceinline__ void gather_gradients(int fd_scheme, const Reader &at
       r2e = at.rho(2 * ex(a), 2 * ey(a), C2e);
       p2e = at.p(2 * ex(a), 2 * ey(a));
     }
+#pragma unroll
     for (int j = 0; j < 3; ++j) n.dC[j][a] = dir_deriv(fd_scheme, Cn[o][j], Cn[0][j], Cn[a][j], C2e[j]);
     n.drho[a] = dir_deriv(fd_scheme, rn[o], rn[0], rn[a], r2e);
     n.dp[a] = dir_deriv(fd_scheme, pn[o], pn[0], pn[a], p2e);
