@@ -69,7 +69,14 @@ __device__ __forceinline__ int i1(int lx, int ly) { return (ly + 1) * (TX + 2) +
 // 32 columns (pop_index), then the planar FP32 P plane, inside the space of the
 // 9 FP32 planes.
 // NT threads per CTA (NT >= TX * TY); NT close to the size of R1 lets the
-// heaviest stage run in one pass.
+// heaviest stage run in one pass.  Where every stage is one pass (NT >= the size of
+// R3: the small tiles of small lattices, which leave SMs idle and wait for latency
+// only), the g of a thread's stage-1 node and the previous tau of its stage-2 node are
+// requested with the stage-0 loads, so that a tile waits for memory once and not three
+// times: 64 x 128 with 16 x 4 tiles and 224 threads 3.7 us per step, with 32 x 8 tiles
+// 5.2 us, with the row sweep 6.2 us (GB300, replayed graph).  The tiles of two or more
+// passes keep the loads where they are used: with the early loads 32x8/352/3 ran 1 %
+// slower (200 x 400: 9.16 -> 9.29 us).
 template <int TX, int TY, int NH, int FORM, int NT>
 __device__ __forceinline__ void fused_tile(const DevParams &P, const FusedBuffers &B, int x0, int y0,
                                            Smem<TX, TY, NH> &s) {
@@ -77,6 +84,18 @@ __device__ __forceinline__ void fused_tile(const DevParams &P, const FusedBuffer
   const int tid = threadIdx.x;
   const long long plane = P.plane;
   const int nx = P.nx, ny = P.ny, per = P.periodic_y, pitch = P.pitch;
+
+  constexpr bool EARLY = NT >= S::N3;
+  float g_early[9], tau_early = 0.f;
+  if constexpr (EARLY) {
+    const int lx2 = tid % S::W2 - 2, gy2 = y0 + tid / S::W2 - 2, lx1 = tid % S::W1 - 1, gy1 = y0 + tid / S::W1 - 1;
+    if (tid < S::N2 && (per || (gy2 >= 0 && gy2 < ny)))
+      load_populations<FORM>(P, B, plane,
+                             (long long)(per ? wrap_periodic(gy2, ny) : gy2) * pitch + wrap_periodic(x0 + lx2, nx),
+                             g_early);
+    if (tid < S::N1 && (per || (gy1 >= 0 && gy1 < ny)))
+      tau_early = B.tau_in[(long long)(per ? wrap_periodic(gy1, ny) : gy1) * pitch + wrap_periodic(x0 + lx1, nx)];
+  }
 
   // ---- stage 0: order parameters and density on R3
   for (int q = tid; q < S::N3; q += NT) {
@@ -97,7 +116,12 @@ __device__ __forceinline__ void fused_tile(const DevParams &P, const FusedBuffer
     if (!per && (gy < 0 || gy >= ny)) continue;
     const long long k = (long long)(per ? wrap_periodic(gy, ny) : gy) * pitch + wrap_periodic(x0 + lx, nx);
     float g[9];
-    load_populations<FORM>(P, B, plane, k, g);
+    if constexpr (EARLY) {
+#pragma unroll
+      for (int a = 0; a < 9; ++a) g[a] = g_early[a];
+    } else {
+      load_populations<FORM>(P, B, plane, k, g);
+    }
     float cn[NH][9], rn[9];
     const int c0 = i3<TX>(lx, ly);
 #pragma unroll
@@ -179,7 +203,7 @@ __device__ __forceinline__ void fused_tile(const DevParams &P, const FusedBuffer
       pair_diff(cn[i], c.DC[i]);
     }
     float hs[NH][9], sv[NH], tn, gd2;
-    node_collide<NH>(P, c, pn, mun, g, B.tau_in[k], hs, sv, tn, gd2);
+    node_collide<NH>(P, c, pn, mun, g, EARLY ? tau_early : B.tau_in[k], hs, sv, tn, gd2);
 #pragma unroll
     for (int a = 0; a < 9; ++a) {
       s.g[a][c2] = g[a];
@@ -290,11 +314,17 @@ static cudaError_t launch_batched_t(const BatchCase *cases, const WorkItem *work
 // single pass) and the minimum resident CTAs per SM passed to the compiler.
 template <int NH, int FORM>
 struct VariantTable {
-  static constexpr int kCount = FORM == 2 ? 2 : (NH == 1 ? 5 : 2);
+  static constexpr int kBatched = FORM == 2 ? 2 : (NH == 1 ? 5 : 2);  // those that batches have too
+  // small tiles for small lattices (not in batches), after the others
+  static constexpr int kSmall = NH == 1 ? 3 : 2;
+  static constexpr int kCount = kBatched + kSmall;
   static const char *name(int v) {
     static const char *n1[5] = {"32x8/352/3", "32x8/448/2", "32x16/640/2", "64x8/704/1", "32x8/352/2"};
     static const char *n2[2] = {"32x8/352/2", "32x8/448/2"};
     static const char *n16[2] = {"32x8/352/3", "32x8/352/2"};
+    static const char *one1[3] = {"16x4/224/2", "32x4/384/2", "32x4/288/3"};
+    static const char *one2[2] = {"16x8/320/2", "32x4/384/1"};
+    if (v >= kBatched) return NH == 1 ? one1[v - kBatched] : one2[v - kBatched];
     return (FORM == 2 && NH == 1) ? n16[v] : (NH == 1 ? n1[v] : n2[v]);
   }
   static void tile(int v, int *tx, int *ty) {
@@ -322,6 +352,16 @@ struct VariantTable {
     }
   }
   static cudaError_t launch(int v, const DevParams &P, const FusedBuffers &B, cudaStream_t s) {
+    if (v >= kBatched) {
+      if constexpr (NH == 1) {
+        if (v == kBatched) return launch_fused_t<16, 4, NH, FORM, 224, 2>(P, B, s);
+        if (v == kBatched + 1) return launch_fused_t<32, 4, NH, FORM, 384, 2>(P, B, s);
+        return launch_fused_t<32, 4, NH, FORM, 288, 3>(P, B, s);
+      } else {
+        if (v == kBatched) return launch_fused_t<16, 8, NH, FORM, 320, 2>(P, B, s);
+        return launch_fused_t<32, 4, NH, FORM, 384, 1>(P, B, s);
+      }
+    }
     if constexpr (FORM == 2 && NH == 1) {
       return v == 1 ? launch_fused_t<32, 8, NH, FORM, 352, 2>(P, B, s) : launch_fused_t<32, 8, NH, FORM, 352, 3>(P, B, s);
     } else if constexpr (NH == 1) {
@@ -360,6 +400,39 @@ const char *fused_variant_name(const DevParams &P, int v) {
   return P.nh == 1 ? VariantTable<1, 0>::name(v) : VariantTable<2, 0>::name(v);
 }
 
+// The configuration a handle starts with, by how much of the GPU the lattice fills.
+// A tile form whose tiles all fit on the device at once beats the row sweep (whose
+// pipeline fill is most of a short segment), the smaller tile the better, until one
+// wave no longer holds them.  Measured per step on a GB300 (152 SMs), population form:
+//   64 x 128   16x4/224 3.7 us (128 tiles)      32x4/384 4.2    32x8/352 5.6    sweep 5.9 us
+//   100 x 200  32x4/384 5.2 us (200 tiles)      16x4/224 5.5+   32x8/352 5.9    sweep 6.8 us
+//   150 x 300  32x4/288 6.5 us (375 tiles)      32x8/352 7.4    sweep 8.0 us
+//   200 x 400  32x8/352 9.2 us (350 tiles)      32x4/288 9.9    sweep 9.7 us
+//   300 x 600  sweep 13.3 us                    32x8/352 14.4 us (750 tiles)
+// Three components: 128 x 128 16x8/320 5.3 us, 32x8/352 7.4, sweep 7.2; 256 x 256 32x8/352
+// 9.4 us (256 tiles), sweep 10.9; 512 x 512 sweep 22.1, 32x8/352 28.3 us.
+int fused_default_variant(const DevParams &P) {
+  static const int sms = [] {
+    int dev = 0, n = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+      return 152;
+    return n;
+  }();
+  auto tiles = [&](int tx, int ty) { return (long long)((P.nx + tx - 1) / tx) * ((P.ny + ty - 1) / ty); };
+  const int ns = sweep_variant_count(P), nb = form_of(P) == 2 || P.nh == 2 ? 2 : 5;
+  if (P.nh == 1) {
+    if (tiles(16, 4) <= sms) return ns + nb;
+    if (tiles(32, 4) <= 2 * sms) return ns + nb + 1;
+    if (tiles(32, 4) <= 3 * sms) return ns + nb + 2;
+    if (tiles(32, 8) <= 3 * sms) return ns;
+  } else {
+    if (tiles(16, 8) <= sms) return ns + nb;
+    if (tiles(32, 8) <= 2 * sms) return ns;
+  }
+  return sweep_default_variant(P, sms);
+}
+
 cudaError_t launch_fused_step(const DevParams &P, const FusedBuffers &B, cudaStream_t s, int v) {
   if (v < 0 || v >= fused_variant_count(P)) v = 0;
   const int ns = sweep_variant_count(P);
@@ -373,7 +446,7 @@ cudaError_t launch_fused_step(const DevParams &P, const FusedBuffers &B, cudaStr
 }
 
 int batched_variant_count(int nh) {
-  return sweep_batched_count(nh) + (nh == 1 ? VariantTable<1, 0>::kCount : VariantTable<2, 0>::kCount);
+  return sweep_batched_count(nh) + (nh == 1 ? VariantTable<1, 0>::kBatched : VariantTable<2, 0>::kBatched);
 }
 
 bool batched_variant_is_sweep(int nh, int v) { return v >= 0 && v < sweep_batched_count(nh); }

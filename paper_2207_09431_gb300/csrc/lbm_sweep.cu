@@ -637,7 +637,25 @@ cudaError_t launch_sweep_t(const DevParams &P, const FusedBuffers &B, cudaStream
 // step / threads / minimum resident CTAs per SM.
 int sweep_variant_count(const DevParams &P) { return P.nh == 1 ? 13 : 4; }
 
-int sweep_default_variant(const DevParams &P) { return P.nh == 1 ? 9 : 0; }
+// Pipeline steps of the slowest CTA slot for strips of tx columns, rs rows per step.
+static int sweep_steps(const DevParams &P, int tx, int rs, int fill, int resident) {
+  const int strips = (P.nx + tx - 1) / tx, len = choose_segment(P.ny, strips, resident, rs, fill);
+  const long long waves = ((long long)strips * ((P.ny + len - 1) / len) + resident - 1) / resident;
+  return (int)(waves * ((len + fill) / rs));
+}
+
+// The sweep a large lattice starts with.  Two components: four-warp strips of 58
+// columns take 0.96 of the time of 160-thread strips of 60 per pipeline step (the
+// fifth warp has almost no items after stage 0), so the 60-column strips are taken where they
+// save more steps than that: 2048 x 4096 (164 against 177 steps: 301 against 305
+// us), not 1024 x 2048 (47 both: 85.5 against 82.1 us), 517 x 1031 (29.1 against 28.0 us).
+// Three components: the shape with fewer steps (512 x 512: 32x4 12 steps, 22.1 us, 64x2
+// 13 steps, 23.2 us; 1024 x 1024: 34 and 33 steps, 75.3 and 70.7 us).
+int sweep_default_variant(const DevParams &P, int sms) {
+  if (P.nh == 1)
+    return 0.96 * sweep_steps(P, 58, 2, fill_rows<2>(), 3 * sms) <= sweep_steps(P, 60, 2, fill_rows<2>(), 3 * sms) ? 11 : 9;
+  return sweep_steps(P, 32, 4, fill_rows<4>(), 2 * sms) < sweep_steps(P, 64, 2, fill_rows<2>(), 2 * sms) ? 1 : 0;
+}
 
 const char *sweep_variant_name(const DevParams &P, int v) {
   static const char *n1[13] = {"64x2/160/3", "32x4/160/3", "128x1/160/2", "64x4/288/2", "64x1/96/5",
