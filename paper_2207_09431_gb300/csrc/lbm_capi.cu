@@ -373,31 +373,26 @@ lbm_status lbm_postprocess(const lbm_params *p, const double raw[15], lbm_obs *o
 lbm_status lbm_observables(lbm_handle *h, lbm_obs *out) {
   if (!h || !out) return LBM_E_INVAL;
   if (!h->initialized) return h->fail(LBM_E_STATE, "observables before initial fields");
-  // C planes (the state itself in the C forms), FP32 populations, then the
-  // sums with u computed per node; no macro-field planes are written
-  lbm::StepBuffers B = h->buffers(h->cur);
-  cudaError_t e = cudaSuccess;
-  const float *g = fp32_populations(h, &e);
-  if (e != cudaSuccess) return h->cuda_fail(e, "FP16 decode");
-  if (B.h_in) lbm::launch_moments(h->dp, B.h_in, B.C, h->stream);
-  e = cudaMemsetAsync(h->acc, 0, 16 * sizeof(double), h->stream);
-  if (e == cudaSuccess) e = cudaMemsetAsync(h->ext, 0x7f, 8 * sizeof(int), h->stream);
-  if (e != cudaSuccess) return h->cuda_fail(e, "observables memset");
-  lbm::launch_observables_direct(h->dp, B.C, g, h->prm.gas_comp, h->acc, h->ext, h->stream);
-  double acc[16];
-  int ext[8];
-  e = cudaGetLastError();
-  if (e == cudaSuccess) e = cudaMemcpyAsync(acc, h->acc, sizeof(acc), cudaMemcpyDeviceToHost, h->stream);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(ext, h->ext, sizeof(ext), cudaMemcpyDeviceToHost, h->stream);
+  // straight from the state, in its stored form; the sums and the extents lie
+  // next to each other (one clear, one copy back)
+  struct {
+    double acc[16];
+    int ext[8];
+  } sums;
+  static_assert(sizeof(sums) == 16 * sizeof(double) + 8 * sizeof(int), "as the arena holds them");
+  cudaError_t e = cudaMemsetAsync(h->acc, 0, sizeof(sums), h->stream);
+  if (e == cudaSuccess)
+    e = lbm::launch_observe(h->dp, h->fused_buffers(h->cur, false), h->prm.gas_comp, h->acc, h->ext, h->stream);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(&sums, h->acc, sizeof(sums), cudaMemcpyDeviceToHost, h->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
   if (e != cudaSuccess) return h->cuda_fail(e, "observables");
   double raw[15];
-  for (int i = 0; i < 11; ++i) raw[i] = acc[i];
-  const bool any = ext[0] != 0x7f7f7f7f;
-  raw[11] = any ? ext[0] : -1.0;
-  raw[12] = any ? -ext[1] : -1.0;
-  raw[13] = any ? ext[2] : -1.0;
-  raw[14] = any ? -ext[3] : -1.0;
+  for (int i = 0; i < 11; ++i) raw[i] = sums.acc[i];
+  const bool any = sums.ext[0] > 0;
+  raw[11] = any ? h->prm.nx - sums.ext[0] : -1.0;
+  raw[12] = any ? sums.ext[1] - 1 : -1.0;
+  raw[13] = any ? h->prm.ny - sums.ext[2] : -1.0;
+  raw[14] = any ? sums.ext[3] - 1 : -1.0;
   lbm_postprocess(&h->prm, raw, out);
   out->step = h->step;
   // centroid y at the first call plus the trapezoidal integral of the rise velocity

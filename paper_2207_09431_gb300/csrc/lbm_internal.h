@@ -14,15 +14,12 @@
 #include "lbm_kernels.h"
 
 namespace lbm {
-// C_i of the population form into the C planes (Eq. 22).
-void launch_moments(const DevParams &P, const float *h, float *C, cudaStream_t s);
 // FP64 observable sums (masses, thresholded masses, sum C_g, C_g-weighted
-// position and velocity, extents of C_g > 0.5) from the C planes and the FP32
-// populations g, with u computed per node as the macro-field kernel computes
-// it; acc (11 doubles) and ext (4 ints: xmin, -xmax, ymin, -ymax) are
-// accumulated with atomics.
-void launch_observables_direct(const DevParams &P, const float *C, const float *g, int gas_comp, double *acc,
-                               int *ext, cudaStream_t s);
+// position and velocity, extents of C_g > 0.5) of the state B.g_in, B.h_in in its
+// stored form; acc (11 doubles) and ext (4 ints: the largest nx - x, x + 1, ny - y,
+// y + 1, 0 where no node exceeds 0.5) are accumulated with atomics from zero.
+cudaError_t launch_observe(const DevParams &P, const FusedBuffers &B, int gas_comp, double *acc, int *ext,
+                           cudaStream_t s);
 // Rows [y0, y1) of nplanes dense FP64 planes into pitched FP32 planes.
 cudaError_t launch_planes_from_f64_rows(const DevParams &P, const double *src, float *dst, int nplanes, int y0,
                                         int y1, cudaStream_t s);

@@ -623,13 +623,6 @@ __global__ void k_init(DevParams P, const float *__restrict__ Cf, const float *_
   tau[k] = tau_mix(P, n.C[0], n.C[1], n.C[2], tau1);
 }
 
-// Observable sums (Sec. 3.1; Eq. 43-44 inputs) in FP64: acc[0..10] = M1..3,
-// M1..3 above 0.5, A, sum C_g x, sum C_g y, sum C_g ux, sum C_g uy; ext[0..3] =
-// xmin, -xmax, ymin, -ymax of C_g > 0.5.  Each thread walks rows (a block per
-// row, grid-stride) accumulating its nodes, then warp shuffles, one
-// shared-memory pass per block and one atomic per block and quantity.
-constexpr int kObsThreads = 256;
-
 // Dense FP64 host-layout planes (ny x nx each) into pitched FP32 planes, one
 // thread per column of the pitch (the padding columns get 0); FP64 -> FP32
 // rounds to nearest, as a host conversion does.
@@ -666,76 +659,121 @@ struct CompSum {
 // one FP64 addition per node and quantity bound the kernel.
 constexpr int kObsRun = 16;
 
-// The observable sums straight from the state: C from the C planes, u
-// computed at each node as k_fields computes it (fields_core), without
-// writing the macro fields.
-template <int NH>
-__global__ void __launch_bounds__(kObsThreads) k_obs_direct(DevParams P, const float *__restrict__ Cf,
-                                                            const float *__restrict__ g, int gas_comp,
-                                                            double *acc, int *ext) {
-  double v[11];
+// Observable sums (Sec. 3.1; Eq. 43-44 inputs) in FP64: acc[0..10] = M1..3,
+// M1..3 above 0.5, A, sum C_g x, sum C_g y, sum C_g ux, sum C_g uy; ext[0..3] =
+// the largest nx - x, x + 1, ny - y, y + 1 of C_g > 0.5 (0: none).  Both zeroed before.
+// Straight from the state in its stored form: a CTA walks tiles of 32 x 8 nodes
+// with C and rho of the tile and its one-node ring in shared memory (two buffers, one
+// barrier per tile), u computed per node by fields_math.  Each state value is read
+// once (the ring's again, from L2), where a pass that wrote C planes and 9-point reads
+// of them through L1 took 391 us at 2048 x 4096 per lbm_observables, and now 232 us (72 B/node at
+// the measured HBM rate: 90 us; bound by the issue of a node's about 600
+// instructions).  Sums: warp shuffles, one shared-memory pass per block, one atomic
+// per block and quantity.
+constexpr int kObsThreads = 256;
+template <int NH, int FORM>
+__global__ void __launch_bounds__(kObsThreads, 3) k_observe(DevParams P, FusedBuffers B, int gas_comp, double *acc,
+                                                            int *ext) {
+  constexpr int TX = 32, TY = 8, W = TX + 2, N = W * (TY + 2);
+  static_assert(TX * TY == kObsThreads, "a thread per node");
+  __shared__ float sC[2][NH][N], srho[2][N];
+  const int t = threadIdx.x, tx = t % TX, ty = t / TX;
+  // the FP64 totals are touched once per run of nodes and wait in shared memory
+  __shared__ double total[11][kObsThreads];
   CompSum r[11];
+#pragma unroll
   for (int q = 0; q < 11; ++q) {
-    v[q] = 0.0;
+    total[q][t] = 0.0;
     r[q] = {0.f, 0.f};
   }
   int run = 0;
   auto flush = [&]() {
+#pragma unroll
     for (int q = 0; q < 11; ++q) {
-      v[q] += (double)r[q].s + (double)r[q].c;
+      total[q][t] += (double)r[q].s + (double)r[q].c;
       r[q] = {0.f, 0.f};
     }
     run = 0;
   };
-  int e[4] = {0x7fffffff, 0x7fffffff, 0x7fffffff, 0x7fffffff};
-  for (int y = blockIdx.x; y < P.ny; y += gridDim.x) {
-    for (int x = threadIdx.x; x < P.nx; x += blockDim.x) {
-      const long long k = node_index(P, x, y);
-      NodeCtx n;
-      float Cn[9][3], rn[9], ga[9], m0;
-      fields_core<NH, false>(P, Cf, g, x, y, k, n, Cn, rn, ga, m0);
-      for (int i = 0; i < 3; ++i) {
-        r[i].add(n.C[i]);
-        r[3 + i].add(n.C[i] > 0.5f ? n.C[i] : 0.0f);
+  int e[4] = {0, 0, 0, 0};
+  const int cols = (P.nx + TX - 1) / TX, tiles = cols * ((P.ny + TY - 1) / TY);
+  int buf = 0;
+  for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x, buf ^= 1) {
+    const int x0 = tile % cols * TX, y0 = tile / cols * TY, x = x0 + tx, y = y0 + ty;
+    const bool mine = x < P.nx && y < P.ny;
+    const bool inside = x0 >= 1 && y0 >= 1 && x0 + TX + 1 <= P.nx && y0 + TY + 1 <= P.ny;
+    float ga[9];
+    if (mine) load_populations<FORM>(P, B, P.plane, node_index(P, x, y), ga);
+#pragma unroll
+    for (int k = 0; k < (N + kObsThreads - 1) / kObsThreads; ++k) {
+      const int q = t + k * kObsThreads;
+      if (q < N) {
+        const int xq = x0 + q % W - 1, yq = y0 + q / W - 1;
+        float c[NH];
+        load_order_parameters<NH, FORM>(B, P.plane, inside ? node_index(P, xq, yq) : tile_node(P, xq, yq), c);
+#pragma unroll
+        for (int i = 0; i < NH; ++i) sC[buf][i][q] = c[i];
+        const float c1 = NH == 2 ? c[NH - 1] : 0.0f;
+        srho[buf][q] = rho_of(P, c[0], c1, 1.0f - c[0] - c1);
       }
-      // C of the gas component, selected without indexing (keeps n in registers)
-      const float cg = gas_comp == 1 ? n.C[0] : (gas_comp == 2 ? n.C[1] : n.C[2]);
-      r[6].add(cg);
-      r[7].add_prod(cg, (float)x);  // x, y < 2^24: exact in FP32
-      r[8].add_prod(cg, (float)y);
-      r[9].add_prod(cg, n.ux);
-      r[10].add_prod(cg, n.uy);
-      if (++run == kObsRun) flush();
-      if (cg > 0.5f) {
-        e[0] = min(e[0], x);
-        e[1] = min(e[1], -x);
-        e[2] = min(e[2], y);
-        e[3] = min(e[3], -y);
-      }
+    }
+    __syncthreads();
+    if (!mine) continue;
+    NodeCtx n;
+    float Cn[9][3], rn[9], m0;
+#pragma unroll
+    for (int a = 0; a < 9; ++a) {
+      const int q = (ty + 1 + ey(a)) * W + tx + 1 + ex(a);
+      Cn[a][0] = sC[buf][0][q];
+      Cn[a][1] = NH == 2 ? sC[buf][NH - 1][q] : 0.0f;
+      Cn[a][2] = 1.0f - Cn[a][0] - Cn[a][1];
+      rn[a] = srho[buf][q];
+    }
+    fields_math<false>(P, n, Cn, rn, ga, m0);
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      r[i].add(n.C[i]);
+      r[3 + i].add(n.C[i] > 0.5f ? n.C[i] : 0.0f);
+    }
+    // C of the gas component, selected without indexing (keeps n in registers)
+    const float cg = gas_comp == 1 ? n.C[0] : (gas_comp == 2 ? n.C[1] : n.C[2]);
+    r[6].add(cg);
+    r[7].add_prod(cg, (float)x);  // x, y < 2^24: exact in FP32
+    r[8].add_prod(cg, (float)y);
+    r[9].add_prod(cg, n.ux);
+    r[10].add_prod(cg, n.uy);
+    if (++run == kObsRun) flush();
+    if (cg > 0.5f) {
+      e[0] = max(e[0], P.nx - x);
+      e[1] = max(e[1], x + 1);
+      e[2] = max(e[2], P.ny - y);
+      e[3] = max(e[3], y + 1);
     }
   }
   flush();
   for (int off = 16; off > 0; off >>= 1) {
-    for (int q = 0; q < 11; ++q) v[q] += __shfl_down_sync(0xffffffffu, v[q], off);
-    for (int q = 0; q < 4; ++q) e[q] = min(e[q], __shfl_down_sync(0xffffffffu, e[q], off));
+#pragma unroll
+    for (int q = 0; q < 4; ++q) e[q] = max(e[q], __shfl_down_sync(0xffffffffu, e[q], off));
   }
-  __shared__ double sv[kObsThreads / 32][11];
   __shared__ int se[kObsThreads / 32][4];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int lane = t & 31, warp = t >> 5;
   if (lane == 0) {
-    for (int q = 0; q < 11; ++q) sv[warp][q] = v[q];
+#pragma unroll
     for (int q = 0; q < 4; ++q) se[warp][q] = e[q];
   }
   __syncthreads();
-  if (threadIdx.x < 11) {
-    double t = 0.0;
-    for (int w = 0; w < kObsThreads / 32; ++w) t += sv[w][threadIdx.x];
-    atomicAdd(&acc[threadIdx.x], t);
-  } else if (threadIdx.x >= 32 && threadIdx.x < 36) {
-    const int q = threadIdx.x - 32;
-    int m = 0x7fffffff;
-    for (int w = 0; w < kObsThreads / 32; ++w) m = min(m, se[w][q]);
-    if (m != 0x7fffffff) atomicMin(&ext[q], m);
+  // the FP64 adder runs at a small fraction of the FP32 rate: a tree over shared memory
+  // fills its lanes, where warp shuffles take five additions of every thread's eleven sums
+  for (int w = kObsThreads / 2; w > 0; w >>= 1) {
+    for (int i = t; i < 11 * w; i += kObsThreads) total[i / w][i & (w - 1)] += total[i / w][(i & (w - 1)) + w];
+    __syncthreads();
+  }
+  if (t < 11) {
+    atomicAdd(&acc[t], total[t][0]);
+  } else if (t >= 32 && t < 36) {
+    int m = 0;
+    for (int w = 0; w < kObsThreads / 32; ++w) m = max(m, se[w][t - 32]);
+    if (m > 0) atomicMax(&ext[t - 32], m);
   }
 }
 
@@ -798,19 +836,22 @@ void launch_init_rows(const DevParams &P, const StepBuffers &B, int y0, int y1, 
 
 void launch_init(const DevParams &P, const StepBuffers &B, cudaStream_t s) { launch_init_rows(P, B, 0, P.ny, s); }
 
-void launch_moments(const DevParams &P, const float *h, float *C, cudaStream_t s) {
-  const dim3 blk(32, 8);
-  k_moments<<<node_grid(P, blk), blk, 0, s>>>(P, h, C);
+cudaError_t launch_observe(const DevParams &P, const FusedBuffers &B, int gas_comp, double *acc, int *ext,
+                           cudaStream_t s) {
+  const long long tiles = (long long)((P.nx + 31) / 32) * ((P.ny + 7) / 8);
+  const int cap = tiles < 912 ? 228 : 456;
+  const int blocks = tiles < cap ? (int)tiles : cap;  // three CTAs per SM, fewer where each would have one tile
+  const int form = P.g16 ? 2 : (P.collapse_h ? 1 : 0);
+  if (P.nh == 1) {
+    if (form == 2) k_observe<1, 2><<<blocks, kObsThreads, 0, s>>>(P, B, gas_comp, acc, ext);
+    else if (form == 1) k_observe<1, 1><<<blocks, kObsThreads, 0, s>>>(P, B, gas_comp, acc, ext);
+    else k_observe<1, 0><<<blocks, kObsThreads, 0, s>>>(P, B, gas_comp, acc, ext);
+  } else {
+    if (form == 2) k_observe<2, 2><<<blocks, kObsThreads, 0, s>>>(P, B, gas_comp, acc, ext);
+    else if (form == 1) k_observe<2, 1><<<blocks, kObsThreads, 0, s>>>(P, B, gas_comp, acc, ext);
+    else k_observe<2, 0><<<blocks, kObsThreads, 0, s>>>(P, B, gas_comp, acc, ext);
+  }
+  return cudaGetLastError();
 }
-
-void launch_observables_direct(const DevParams &P, const float *C, const float *g, int gas_comp, double *acc,
-                               int *ext, cudaStream_t s) {
-  const int blocks = P.ny < 1216 ? P.ny : 1216;  // 8 per SM on 152 SMs, at most one per row
-  if (P.nh == 1)
-    k_obs_direct<1><<<blocks, kObsThreads, 0, s>>>(P, C, g, gas_comp, acc, ext);
-  else
-    k_obs_direct<2><<<blocks, kObsThreads, 0, s>>>(P, C, g, gas_comp, acc, ext);
-}
-
 
 }  // namespace lbm
