@@ -152,7 +152,7 @@ lbm_status lbm_create(const lbm_params *p, void *dev_arena, size_t arena_bytes, 
  * periodic axes), uniform noise in [-noise_amp, noise_amp] from SplitMix64 at
  * counter (comp - 1) * nx * ny + node is added to every disc component, the
  * matrix takes the rest; then as lbm_set_fields with p = u = 0.  Computed in
- * FP64 on the host, uploaded, equilibria built on the device. */
+ * FP64 on the device. */
 lbm_status lbm_init_bubbles(lbm_handle *h, const lbm_bubble *bubbles, int nb, unsigned long long seed,
                             double noise_amp);
 
@@ -160,12 +160,12 @@ lbm_status lbm_init_bubbles(lbm_handle *h, const lbm_bubble *bubbles, int nb, un
  * planes (C1, then C2); p, ux, uy may be NULL for zero.  Populations are the
  * modified equilibria of Eq. 16 and Eq. 20; tau uses a zero strain rate.  The
  * doubles are copied to the device as they are (through the spare population
- * buffer) and rounded to FP32 there; page-locked host memory makes the copy
- * faster.  With FP32 populations, at least 64 rows and a stream that is not
- * being captured, C goes up in row chunks on a second stream that the handle
+ * buffer and scratch planes) and rounded to FP32 there; page-locked host memory
+ * makes the copy faster.  With at least 64 rows and a stream that is not being
+ * captured, the fields go up in row chunks on a second stream that the handle
  * creates on first use (and destroys with the handle), overlapped with the
- * conversion and the equilibria on the handle's stream.  Synchronises the
- * stream; returns when every copy is done. */
+ * equilibria on the handle's stream.  Synchronises the stream; returns when
+ * every copy is done. */
 lbm_status lbm_set_fields(lbm_handle *h, const double *C, const double *p, const double *ux,
                           const double *uy);
 

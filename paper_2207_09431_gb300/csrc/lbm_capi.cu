@@ -17,55 +17,32 @@
 
 #include "lbm_internal.h"
 
-// Copies nplanes host planes (dense ny x nx doubles) into pitched device FP32
-// planes: the doubles go to the device as they are, staged in the spare
-// population buffer g[1] (free until the initial equilibria are built), and a
-// kernel converts them; a NULL source sets the planes to zero.  Enqueued on
-// the handle's stream; the caller synchronises.
-static cudaError_t upload_planes(lbm_handle *h, float *dst, const double *src, int nplanes) {
-  const size_t plane_bytes = h->L.plane_bytes;
-  if (!src) return cudaMemsetAsync(dst, 0, (size_t)nplanes * plane_bytes, h->stream);
-  const size_t bytes = (size_t)nplanes * h->prm.nx * h->prm.ny * sizeof(double);
-  if (bytes > 9 * plane_bytes) return cudaErrorInvalidValue;  // cannot happen: 2 planes of doubles < 9 of floats
-  double *staging = reinterpret_cast<double *>(h->g[1]);
-  cudaError_t e = cudaMemcpyAsync(staging, src, bytes, cudaMemcpyHostToDevice, h->stream);
-  if (e == cudaSuccess) e = lbm::launch_planes_from_f64(h->dp, staging, dst, nplanes, h->stream);
+// Fields go to the host as dense doubles, converted on the device in the spare
+// population buffer (free between steps; four dense planes of doubles fit) and copied
+// straight into the caller's array.
+static cudaError_t download_planes(lbm_handle *h, const float *src, double *dst, int nplanes, int kind = lbm::kPlane) {
+  const size_t N = (size_t)h->prm.nx * h->prm.ny;
+  double *dense = reinterpret_cast<double *>(h->g[1 - h->cur]);
+  cudaError_t e = lbm::launch_planes_to_f64(h->dp, h->prm.rho, src, kind, nplanes, dense, h->stream);
+  if (e == cudaSuccess)
+    e = cudaMemcpyAsync(dst, dense, nplanes * N * sizeof(double), cudaMemcpyDeviceToHost, h->stream);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
   return e;
 }
 
-// Copies nplanes pitched device planes into dense host doubles.
-static cudaError_t download_planes(lbm_handle *h, const float *src, double *dst, int nplanes) {
-  const int nx = h->prm.nx, ny = h->prm.ny, pitch = h->dp.pitch;
-  h->stage.assign((size_t)nplanes * h->plane_floats(), 0.0f);
-  for (int q = 0; q < nplanes; ++q) {
-    cudaError_t e = cudaMemcpyAsync(h->stage.data() + (size_t)q * h->plane_floats(),
-                                    src + (size_t)q * (h->L.plane_bytes / sizeof(float)),
-                                    h->plane_floats() * sizeof(float), cudaMemcpyDeviceToHost, h->stream);
-    if (e != cudaSuccess) return e;
+// The nq planes of a device population array, plane after plane.
+static cudaError_t download_pops(lbm_handle *h, const float *src, double *dst, int nq, bool g16) {
+  const size_t N = (size_t)h->prm.nx * h->prm.ny;
+  double *dense = reinterpret_cast<double *>(h->g[1 - h->cur]);
+  cudaError_t e = cudaSuccess;
+  for (int q0 = 0; q0 < nq && e == cudaSuccess; q0 += 4) {
+    const int q1 = std::min(nq, q0 + 4);
+    e = lbm::launch_pops_to_f64(h->dp, src, q0, q1, nq, g16, dense, h->stream);
+    if (e == cudaSuccess)
+      e = cudaMemcpyAsync(dst + q0 * N, dense, (q1 - q0) * N * sizeof(double), cudaMemcpyDeviceToHost, h->stream);
   }
-  cudaError_t e = cudaStreamSynchronize(h->stream);
-  if (e != cudaSuccess) return e;
-  for (int q = 0; q < nplanes; ++q)
-    for (int y = 0; y < ny; ++y)
-      for (int x = 0; x < nx; ++x)
-        dst[((size_t)q * ny + y) * nx + x] = h->stage[(size_t)q * h->plane_floats() + (size_t)y * pitch + x];
-  return cudaSuccess;
-}
-
-// Copies a device population array (nq planes interleaved in blocks of 32
-// columns, lbm::pop_index) into dense host doubles, plane after plane.
-static cudaError_t download_pops(lbm_handle *h, const float *src, double *dst, int nq) {
-  const int nx = h->prm.nx, ny = h->prm.ny, pitch = h->dp.pitch;
-  const size_t n = (size_t)nq * ny * pitch;
-  h->stage.assign(n, 0.0f);
-  cudaError_t e = cudaMemcpyAsync(h->stage.data(), src, n * sizeof(float), cudaMemcpyDeviceToHost, h->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
-  if (e != cudaSuccess) return e;
-  for (int q = 0; q < nq; ++q)
-    for (int y = 0; y < ny; ++y)
-      for (int x = 0; x < nx; ++x)
-        dst[((size_t)q * ny + y) * nx + x] = h->stage[lbm::pop_index((long long)y * pitch + x, q, nq)];
-  return cudaSuccess;
+  return e;
 }
 
 extern "C" {
@@ -126,13 +103,11 @@ lbm_status lbm_create(const lbm_params *p, void *dev_arena, size_t arena_bytes, 
   return LBM_OK;
 }
 
-// Whether lbm_set_fields may overlap the upload of C with the conversion and
-// the initial equilibria: FP32 populations (the FP16 form computes its
-// equilibria into the staging buffer), chunks of at least 16 rows (the
-// equilibria read two rows beyond their own), and a stream that is not being
-// captured.  The copy stream and its events are created on first use.
+// Whether lbm_set_fields may overlap the upload with the initial equilibria: chunks
+// of at least 16 rows (the equilibria read two rows beyond their own), and a stream
+// that is not being captured.  The copy stream and its events are created on first use.
 static bool upload_overlappable(lbm_handle *h) {
-  if (h->dp.g16 || h->prm.ny < 16 * lbm_handle::kUploadChunks) return false;
+  if (h->prm.ny < 16 * lbm_handle::kUploadChunks) return false;
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
   if (cudaStreamIsCapturing(h->stream, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) return false;
   if (!h->copy_stream && cudaStreamCreateWithFlags(&h->copy_stream, cudaStreamNonBlocking) != cudaSuccess) {
@@ -147,73 +122,61 @@ static bool upload_overlappable(lbm_handle *h) {
   return true;
 }
 
-// C goes up in row chunks on the copy stream; the handle's stream converts each
-// chunk once it has arrived and computes the equilibria of the rows whose
-// two-row neighbourhood is converted (those of the first chunk last under
-// periodic y, where they read the last rows).  Same node values as one upload.
-static cudaError_t upload_and_init_overlapped(lbm_handle *h, const double *C, int nh, const lbm::StepBuffers &B) {
+// FP64 fields on the device, dense: C in the spare population buffer g[1] (free
+// until the first step), p, ux and uy in the scratch planes mu .. uy, which lie next
+// to each other (six FP32 planes hold three of doubles).
+struct StagedFields {
+  double *C, *f[3];
+  explicit StagedFields(const lbm_handle *h) : C(reinterpret_cast<double *>(h->g[1])) {
+    for (int q = 0; q < 3; ++q) f[q] = reinterpret_cast<double *>(reinterpret_cast<char *>(h->mu) + 2 * q * h->L.plane_bytes);
+  }
+};
+
+// Equilibria of rows [y0, y1) into buffer 0 from the staged fields.
+static cudaError_t init_rows(lbm_handle *h, const StagedFields &st, const bool given[3], int y0, int y1) {
+  return lbm::launch_init_rows(h->dp, st.C, given[0] ? st.f[0] : nullptr, given[1] ? st.f[1] : nullptr,
+                               given[2] ? st.f[2] : nullptr, h->g[0], h->h[0], h->tau[0], y0, y1, h->stream);
+}
+
+// The fields go up in row chunks on the copy stream; the handle's stream computes the
+// equilibria of the rows whose two-row neighbourhood has arrived (those of the first
+// chunk last under periodic y, where they read the last rows).  Same node values as
+// one upload.
+static cudaError_t upload_and_init_overlapped(lbm_handle *h, const StagedFields &st, const double *C,
+                                              const double *const f[3], const bool given[3]) {
   constexpr int n = lbm_handle::kUploadChunks;
-  const int nx = h->prm.nx, ny = h->prm.ny, rows = (ny + n - 1) / n;
+  const int nh = h->prm.ncomp - 1, nx = h->prm.nx, ny = h->prm.ny, rows = (ny + n - 1) / n;
   const bool per = h->prm.periodic_y != 0;
-  double *staging = reinterpret_cast<double *>(h->g[1]);
-  // the staging buffer is free once the uploads before on the stream are done
+  // the staging buffers are free once the work before on the stream is done
   cudaError_t e = cudaEventRecord(h->upload_ev[n], h->stream);
   if (e == cudaSuccess) e = cudaStreamWaitEvent(h->copy_stream, h->upload_ev[n], 0);
   for (int c = 0; c < n && e == cudaSuccess; ++c) {
     const int y0 = c * rows, y1 = std::min(ny, y0 + rows);
+    const size_t bytes = (size_t)(y1 - y0) * nx * sizeof(double);
     for (int q = 0; q < nh && e == cudaSuccess; ++q) {
       const size_t off = ((size_t)q * ny + y0) * nx;
-      e = cudaMemcpyAsync(staging + off, C + off, (size_t)(y1 - y0) * nx * sizeof(double), cudaMemcpyHostToDevice,
-                          h->copy_stream);
+      e = cudaMemcpyAsync(st.C + off, C + off, bytes, cudaMemcpyHostToDevice, h->copy_stream);
     }
+    for (int q = 0; q < 3 && e == cudaSuccess; ++q)
+      if (given[q])
+        e = cudaMemcpyAsync(st.f[q] + (size_t)y0 * nx, f[q] + (size_t)y0 * nx, bytes, cudaMemcpyHostToDevice,
+                            h->copy_stream);
     if (e == cudaSuccess) e = cudaEventRecord(h->upload_ev[c], h->copy_stream);
   }
   for (int c = 0; c < n && e == cudaSuccess; ++c) {
-    const int y0 = c * rows, y1 = std::min(ny, y0 + rows);
     e = cudaStreamWaitEvent(h->stream, h->upload_ev[c], 0);
-    if (e == cudaSuccess) e = lbm::launch_planes_from_f64_rows(h->dp, staging, h->C, nh, y0, y1, h->stream);
-    if (e == cudaSuccess && c >= 1 && (c >= 2 || !per)) {
-      lbm::launch_init_rows(h->dp, B, (c - 1) * rows, c * rows, h->stream);
-      e = cudaGetLastError();
-    }
+    if (e == cudaSuccess && c >= 1 && (c >= 2 || !per)) e = init_rows(h, st, given, (c - 1) * rows, c * rows);
   }
-  if (e == cudaSuccess) {
-    lbm::launch_init_rows(h->dp, B, (n - 1) * rows, ny, h->stream);
-    if (per) lbm::launch_init_rows(h->dp, B, 0, rows, h->stream);
-    e = cudaGetLastError();
-  }
+  if (e == cudaSuccess) e = init_rows(h, st, given, (n - 1) * rows, ny);
+  if (e == cudaSuccess && per) e = init_rows(h, st, given, 0, rows);
   return e;
 }
 
-lbm_status lbm_set_fields(lbm_handle *h, const double *C, const double *p, const double *ux, const double *uy) {
-  if (!h) return LBM_E_INVAL;
-  if (!C) return h->fail(LBM_E_INVAL, "C is NULL");
-  const int nh = h->prm.ncomp - 1;
-  const bool overlap = upload_overlappable(h);
-  cudaError_t e = overlap ? cudaSuccess : upload_planes(h, h->C, C, nh);
-  if (e == cudaSuccess) e = upload_planes(h, h->p, p, 1);
-  if (e == cudaSuccess) e = upload_planes(h, h->ux, ux, 1);
-  if (e == cudaSuccess) e = upload_planes(h, h->uy, uy, 1);
-  if (e != cudaSuccess) return h->cuda_fail(e, "lbm_set_fields upload");
-  // equilibria into buffer 0
-  lbm::StepBuffers B = h->buffers(1);  // *_out of buffer index 1 is buffer 0
-  if (h->dp.g16) B.g_out = h->g[1];    // FP32 equilibria into the spare, encoded below
-  if (h->prm.collapse_h) {
-    B.C = h->C;
-    B.h_out = nullptr;
-  }
-  if (overlap) {
-    e = upload_and_init_overlapped(h, C, nh, B);
-  } else {
-    lbm::launch_init(h->dp, B, h->stream);
-    e = cudaGetLastError();
-  }
-  // the C state: the converted order parameters
-  if (e == cudaSuccess && h->prm.collapse_h)
-    e = cudaMemcpyAsync(h->h[0], h->C, (size_t)nh * h->L.plane_bytes, cudaMemcpyDeviceToDevice, h->stream);
-  if (e == cudaSuccess && h->dp.g16) e = lbm::launch_g16_encode(h->dp, h->g[1], h->g[0], h->stream);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
-  if (e != cudaSuccess) return h->cuda_fail(e, "lbm_set_fields init kernel");
+// The state that the staged fields (or those still to be uploaded) have become.
+static lbm_status fields_set(lbm_handle *h, cudaError_t e) {
+  const cudaError_t done = cudaStreamSynchronize(h->stream);
+  if (e == cudaSuccess) e = done;
+  if (e != cudaSuccess) return h->cuda_fail(e, "lbm_set_fields");
   h->cur = 0;
   h->initialized = true;
   h->step = 0;
@@ -222,41 +185,48 @@ lbm_status lbm_set_fields(lbm_handle *h, const double *C, const double *p, const
   return LBM_OK;
 }
 
+lbm_status lbm_set_fields(lbm_handle *h, const double *C, const double *p, const double *ux, const double *uy) {
+  if (!h) return LBM_E_INVAL;
+  if (!C) return h->fail(LBM_E_INVAL, "C is NULL");
+  const int nh = h->prm.ncomp - 1;
+  const StagedFields st(h);
+  const double *const f[3] = {p, ux, uy};
+  const bool given[3] = {p != nullptr, ux != nullptr, uy != nullptr};
+  if (upload_overlappable(h)) return fields_set(h, upload_and_init_overlapped(h, st, C, f, given));
+  const size_t bytes = (size_t)h->prm.nx * h->prm.ny * sizeof(double);
+  cudaError_t e = cudaMemcpyAsync(st.C, C, nh * bytes, cudaMemcpyHostToDevice, h->stream);
+  for (int q = 0; q < 3 && e == cudaSuccess; ++q)
+    if (given[q]) e = cudaMemcpyAsync(st.f[q], f[q], bytes, cudaMemcpyHostToDevice, h->stream);
+  if (e == cudaSuccess) e = init_rows(h, st, given, 0, h->prm.ny);
+  return fields_set(h, e);
+}
+
 lbm_status lbm_init_bubbles(lbm_handle *h, const lbm_bubble *bubbles, int nb, unsigned long long seed,
                             double noise_amp) {
   if (!h) return LBM_E_INVAL;
   if (nb < 0 || (nb > 0 && !bubbles)) return h->fail(LBM_E_INVAL, "bad bubble list");
-  const int nx = h->prm.nx, ny = h->prm.ny, nh = h->prm.ncomp - 1;
-  const size_t n = (size_t)nx * ny;
-  std::vector<double> comp[2] = {std::vector<double>(n, 0.0), std::vector<double>(n, 0.0)};  // comps 2, 3
+  const int nh = h->prm.ncomp - 1;
   bool used[2] = {false, false};
   for (int b = 0; b < nb; ++b) {
     const int c = bubbles[b].comp;
     if (c < 2 || c > 3 || (nh == 1 && c != 3)) return h->fail(LBM_E_INVAL, "disc component must be 3 (or 2 with ncomp 3)");
     used[c - 2] = true;
-    for (int y = 0; y < ny; ++y)
-      for (int x = 0; x < nx; ++x) {
-        double dx = std::fabs(x - bubbles[b].cx), dy = std::fabs(y - bubbles[b].cy);
-        if (dx > 0.5 * nx) dx = nx - dx;
-        if (h->prm.periodic_y && dy > 0.5 * ny) dy = ny - dy;
-        const double r = std::sqrt(dx * dx + dy * dy);
-        comp[c - 2][(size_t)y * nx + x] += 0.5 - 0.5 * std::tanh((r - bubbles[b].r) / (0.5 * h->prm.xi));
-      }
   }
-  for (int c = 0; c < 2; ++c) {
-    if (!used[c] || noise_amp == 0.0) continue;
-    for (size_t k = 0; k < n; ++k) {
-      const uint64_t z = splitmix64_at(seed, (uint64_t)(c + 1) * n + k);
-      const double u01 = (double)(z >> 11) * (1.0 / 9007199254740992.0);
-      comp[c][k] += noise_amp * (2.0 * u01 - 1.0);
-    }
+  const StagedFields st(h);
+  cudaError_t e = cudaSuccess;
+  for (int b0 = 0; (b0 < nb || b0 == 0) && e == cudaSuccess; b0 += lbm::kDiscs) {
+    lbm::DiscGroup d{};
+    d.count = std::min(nb - b0, lbm::kDiscs);
+    std::copy(bubbles + b0, bubbles + b0 + d.count, d.disc);
+    d.first = b0 == 0;
+    d.last = b0 + lbm::kDiscs >= nb;
+    d.seed = seed;
+    for (int c = 0; c < 2; ++c) d.noise[c] = used[c] ? noise_amp : 0.0;
+    e = lbm::launch_discs(h->dp, h->prm.xi, d, st.C, h->stream);
   }
-  std::vector<double> Cin((size_t)nh * n);
-  for (size_t k = 0; k < n; ++k) {
-    Cin[k] = 1.0 - comp[0][k] - comp[1][k];
-    if (nh == 2) Cin[n + k] = comp[0][k];
-  }
-  return lbm_set_fields(h, Cin.data(), nullptr, nullptr, nullptr);
+  const bool given[3] = {false, false, false};
+  if (e == cudaSuccess) e = init_rows(h, st, given, 0, h->prm.ny);
+  return fields_set(h, e);
 }
 
 lbm_status lbm_step(lbm_handle *h, long long nsteps) {
@@ -425,48 +395,37 @@ lbm_status lbm_get_field(lbm_handle *h, int id, double *out, size_t n) {
   }
   if (n < need) return h->fail(LBM_E_INVAL, "output buffer too small");
   const size_t pf = h->L.plane_bytes / sizeof(float);
+  // C_i (the state itself in the C forms)
+  auto c_planes = [&]() -> const float * {
+    const lbm::StepBuffers B = h->buffers(h->cur);
+    if (B.h_in) lbm::launch_moments(h->dp, B.h_in, B.C, h->stream);
+    return B.C;
+  };
   cudaError_t e = cudaSuccess;
   switch (id) {
-    case LBM_FIELD_G: {
-      const float *g32 = fp32_populations(h, &e);
-      if (e == cudaSuccess) e = download_pops(h, g32, out, 9);
-      break;
-    }
+    case LBM_FIELD_G: e = download_pops(h, h->g[h->cur], out, 9, h->dp.g16); break;
     case LBM_FIELD_H:
       if (h->prm.collapse_h) return h->fail(LBM_E_STATE, "the collapsed state form stores no h populations");
-      e = download_pops(h, h->h[h->cur], out, 9 * nh);
+      e = download_pops(h, h->h[h->cur], out, 9 * nh, false);
       break;
     case LBM_FIELD_TAU: e = download_planes(h, h->tau[h->cur], out, 1); break;
     case LBM_FIELD_SHEAR: e = download_planes(h, h->shear, out, 1); break;
     case LBM_FIELD_SV: e = download_planes(h, h->SV, out, nh); break;
+    case LBM_FIELD_C1: e = download_planes(h, c_planes(), out, 1); break;
+    case LBM_FIELD_C2:
+      if (nh == 2) e = download_planes(h, c_planes() + pf, out, 1);
+      else std::memset(out, 0, N * sizeof(double));
+      break;
+    case LBM_FIELD_C3: e = download_planes(h, c_planes(), out, 1, lbm::kThird); break;
+    case LBM_FIELD_RHO: e = download_planes(h, c_planes(), out, 1, lbm::kDensity); break;
     default: {
-      lbm_status st = compute_macros(h);
+      const lbm_status st = compute_macros(h);
       if (st != LBM_OK) return st;
-      const float *Cp = h->buffers(h->cur).C;
-      if (id == LBM_FIELD_C1) e = download_planes(h, Cp, out, 1);
-      else if (id == LBM_FIELD_C2) {
-        if (nh == 2) e = download_planes(h, Cp + pf, out, 1);
-        else std::memset(out, 0, N * sizeof(double));
-      } else if (id == LBM_FIELD_C3 || id == LBM_FIELD_RHO) {
-        std::vector<double> c(2 * N, 0.0);
-        e = download_planes(h, Cp, c.data(), nh);
-        if (e == cudaSuccess)
-          for (size_t k = 0; k < N; ++k) {
-            // C3 = 1 - C1 - C2 (Eq. 1); rho by the clipped mixture law (R1)
-            const double C1 = (float)c[k], C2 = nh == 2 ? (float)c[N + k] : 0.0;
-            const double C3 = (double)(1.0f - (float)C1 - (float)C2);
-            if (id == LBM_FIELD_C3) {
-              out[k] = C3;
-            } else {
-              double w[3] = {C1, C2, C3}, s = 0;
-              for (double &v : w) { v = v < 0 ? 0 : (v > 1 ? 1 : v); s += v; }
-              out[k] = (w[0] * h->prm.rho[0] + w[1] * h->prm.rho[1] + w[2] * h->prm.rho[2]) / s;
-            }
-          }
-      } else if (id == LBM_FIELD_P) e = download_planes(h, h->p, out, 1);
-      else if (id == LBM_FIELD_UX) e = download_planes(h, h->ux, out, 1);
-      else if (id == LBM_FIELD_UY) e = download_planes(h, h->uy, out, 1);
-      else e = download_planes(h, h->mu + (size_t)(id - LBM_FIELD_MU1) * pf, out, 1);
+      const float *src = id == LBM_FIELD_P    ? h->p
+                         : id == LBM_FIELD_UX ? h->ux
+                         : id == LBM_FIELD_UY ? h->uy
+                                              : h->mu + (size_t)(id - LBM_FIELD_MU1) * pf;
+      e = download_planes(h, src, out, 1);
     }
   }
   if (e != cudaSuccess) return h->cuda_fail(e, "lbm_get_field");

@@ -479,21 +479,7 @@ cudaError_t launch_batched_step(int nh, int form, const BatchCase *cases, const 
   return VariantTable<2, 0>::launch_batched(v, cases, work, nwork, parity, s);
 }
 
-// Conversions between the FP32 populations and the FORM 2 storage (initial
-// state, field readback), one thread per node.
-__global__ void k_g16_encode(DevParams P, const float *__restrict__ g32, float *__restrict__ g16) {
-  const long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= P.plane) return;
-  float g[9];
-#pragma unroll
-  for (int a = 0; a < 9; ++a) g[a] = g32[pop_index(k, a, 9)];
-  const float Pn = g16_reference(g);
-  g16[(9 * P.plane) / 2 + k] = Pn;
-  __half *gh = reinterpret_cast<__half *>(g16);
-#pragma unroll
-  for (int a = 0; a < 9; ++a) gh[pop_index(k, a, 9)] = g16_encode(g[a], Pn, a, P.g16_scale);
-}
-
+// FP32 populations of the FORM 2 storage (for the macro fields), one thread per node.
 __global__ void k_g16_decode(DevParams P, const float *__restrict__ g16, float *__restrict__ g32) {
   const long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= P.plane) return;
@@ -501,11 +487,6 @@ __global__ void k_g16_decode(DevParams P, const float *__restrict__ g16, float *
   const __half *gh = reinterpret_cast<const __half *>(g16);
 #pragma unroll
   for (int a = 0; a < 9; ++a) g32[pop_index(k, a, 9)] = g16_decode(Pref, gh[pop_index(k, a, 9)], a, P.g16_inv_scale);
-}
-
-cudaError_t launch_g16_encode(const DevParams &P, const float *g32, float *g16, cudaStream_t s) {
-  k_g16_encode<<<(unsigned)((P.plane + 255) / 256), 256, 0, s>>>(P, g32, g16);
-  return cudaGetLastError();
 }
 
 cudaError_t launch_g16_decode(const DevParams &P, const float *g16, float *g32, cudaStream_t s) {

@@ -20,12 +20,31 @@ namespace lbm {
 // y + 1, 0 where no node exceeds 0.5) are accumulated with atomics from zero.
 cudaError_t launch_observe(const DevParams &P, const FusedBuffers &B, int gas_comp, double *acc, int *ext,
                            cudaStream_t s);
-// Rows [y0, y1) of nplanes dense FP64 planes into pitched FP32 planes.
-cudaError_t launch_planes_from_f64_rows(const DevParams &P, const double *src, float *dst, int nplanes, int y0,
-                                        int y1, cudaStream_t s);
-// Initial equilibria (modified, Eq. 14 and 18 at rest of the forcing) of rows
-// [y0, y1); they read C and p up to two rows beyond.
-void launch_init_rows(const DevParams &P, const StepBuffers &B, int y0, int y1, cudaStream_t s);
+// Up to kDiscs initial discs of one launch of a set: the sums so far are in the planes
+// (unless first), the noise amplitudes of components 2 and 3 (0: none) and the matrix come last.
+constexpr int kDiscs = 16;
+struct DiscGroup {
+  lbm_bubble disc[kDiscs];
+  int count, first, last;
+  unsigned long long seed;
+  double noise[2];
+};
+// Discs as dense FP64 planes of C (nh planes of ny x nx, device).
+cudaError_t launch_discs(const DevParams &P, double xi, const DiscGroup &d, double *C, cudaStream_t s);
+// C_i of the population form into the C planes (Eq. 22).
+void launch_moments(const DevParams &P, const float *h, float *C, cudaStream_t s);
+// Device fields as dense FP64 planes (device): nplanes FP32 planes, or C_3 or the
+// density from the C planes; planes [q0, q1) of a population array of nq planes.
+enum { kPlane = 0, kThird = 1, kDensity = 2 };
+cudaError_t launch_planes_to_f64(const DevParams &P, const double rho[3], const float *src, int kind, int nplanes,
+                                 double *dst, cudaStream_t s);
+cudaError_t launch_pops_to_f64(const DevParams &P, const float *src, int q0, int q1, int nq, bool g16, double *dst,
+                               cudaStream_t s);
+// Initial equilibria (modified, Eq. 16 and 20 at zero strain rate) of rows [y0, y1)
+// into a state's buffers in its stored form, from dense FP64 device planes (C:
+// nh planes; p, ux, uy one each or NULL for zero), which are read up to two rows beyond.
+cudaError_t launch_init_rows(const DevParams &P, const double *C, const double *p, const double *ux, const double *uy,
+                             float *g, float *h, float *tau, int y0, int y1, cudaStream_t s);
 }  // namespace lbm
 
 namespace lbm_detail {
@@ -164,14 +183,6 @@ inline lbm::DevParams dev_params(const lbm_params &p) {
   return d;
 }
 
-// SplitMix64 (Steele, Lea and Flood 2014) at counter i: mix(seed + (i+1) gamma).
-inline uint64_t splitmix64_at(uint64_t seed, uint64_t i) {
-  uint64_t z = seed + (i + 1) * 0x9E3779B97F4A7C15ULL;
-  z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ULL;
-  z = (z ^ (z >> 27)) * 0x94D049BB133111EBULL;
-  return z ^ (z >> 31);
-}
-
 }  // namespace lbm_detail
 
 using namespace lbm_detail;
@@ -196,7 +207,6 @@ struct lbm_handle {
   long long prev_step;
   double prev_v, y_int;
   std::string last_error;
-  std::vector<float> stage;  // host staging (pitched FP32 planes)
   // captured runs of kStepGraph steps without diagnostics, one per starting
   // buffer (cur), for the launch configuration they were captured with
   cudaGraphExec_t graph[2] = {nullptr, nullptr};

@@ -94,15 +94,10 @@ cudaError_t launch_sweep_step(const DevParams &P, const FusedBuffers &B, cudaStr
 int fused_variant_count(const DevParams &P);
 const char *fused_variant_name(const DevParams &P, int v);
 cudaError_t launch_fused_step(const DevParams &P, const FusedBuffers &B, cudaStream_t s, int v);
-// FP16 storage (P.g16): g32 holds 9 FP32 planes, g16 the same space as 9 half
-// planes followed by the FP32 plane of the per-node reference sum_a g_a.
-cudaError_t launch_g16_encode(const DevParams &P, const float *g32, float *g16, cudaStream_t s);
+// FP16 storage (P.g16): g16 holds 9 half planes followed by the FP32 plane of the
+// per-node reference sum_a g_a; g32 receives 9 FP32 planes.
 cudaError_t launch_g16_decode(const DevParams &P, const float *g16, float *g32, cudaStream_t s);
 
 void launch_macros(const DevParams &P, const StepBuffers &B, cudaStream_t s);
-void launch_init(const DevParams &P, const StepBuffers &B, cudaStream_t s);
-// nplanes dense FP64 planes (ny x nx each, device) into pitched FP32 planes
-// (plane stride P.plane floats).
-cudaError_t launch_planes_from_f64(const DevParams &P, const double *src, float *dst, int nplanes, cudaStream_t s);
 
 }  // namespace lbm

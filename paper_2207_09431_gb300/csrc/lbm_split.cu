@@ -9,6 +9,7 @@
 // arena.  All arithmetic FP32.  Also the macro fields, the initial equilibria and
 // the observables.
 #include "lbm_device.cuh"
+#include "lbm_internal.h"
 #include "lbm_kernels.h"
 #include "lbm_node.cuh"
 
@@ -61,19 +62,8 @@ struct NodeCtx {
   float dC[3][9], drho[9], dp[9];
 };
 
-// Field values around a node, from the planes.
-struct PlaneReader {
-  const DevParams &P;
-  CReader cr;
-  const float *pf;
-  int x, y;
-  __device__ __forceinline__ void C(int dx, int dy, float c[3]) const { cr.at(shifted(P, x, y, dx, dy), c); }
-  __device__ __forceinline__ float rho(int, int, const float c[3]) const { return rho_of(P, c[0], c[1], c[2]); }
-  __device__ __forceinline__ float p(int dx, int dy) const { return pf[shifted(P, x, y, dx, dy)]; }
-};
-
 // Gathers C (radius 1 or 2), rho (from C), p (radius 1 or 2) around a node.
-// Inlined, so that NodeCtx stays in registers.
+// Inlined and unrolled, so that NodeCtx stays in registers.
 template <typename Reader>
 __device__ __forceinline__ void gather_gradients(int fd_scheme, const Reader &at, NodeCtx &n) {
   float Cn[9][3], rn[9], pn[9];
@@ -245,15 +235,13 @@ __global__ void k_fields(DevParams P, const float *__restrict__ Cf, const float 
 // Row and column whose values stand at (x, y) of a tile and its rings: periodic, or
 // the mirror ghost rows beyond walls and ghost columns beyond the open ends
 // (slots far outside, of ragged tiles, hold some value that nothing reads).
+__device__ __forceinline__ int tile_column(const DevParams &P, int x) {
+  if (!P.open_x) return wrap_periodic(x, P.nx);
+  const int xs = x < 0 ? -1 - x : (x >= P.nx ? 2 * P.nx - 1 - x : x);
+  return xs < 0 ? 0 : (xs >= P.nx ? P.nx - 1 : xs);
+}
 __device__ __forceinline__ long long tile_node(const DevParams &P, int x, int y) {
-  int xs;
-  if (!P.open_x) {
-    xs = wrap_periodic(x, P.nx);
-  } else {
-    xs = x < 0 ? -1 - x : (x >= P.nx ? 2 * P.nx - 1 - x : x);
-    xs = xs < 0 ? 0 : (xs >= P.nx ? P.nx - 1 : xs);
-  }
-  return node_index(P, xs, row_read(y, P.ny, P.periodic_y));
+  return node_index(P, tile_column(P, x), row_read(y, P.ny, P.periodic_y));
 }
 
 // Both step kernels take a tile of 32 x 4 output nodes per CTA and keep the
@@ -584,55 +572,198 @@ __global__ void __launch_bounds__(kCollideThreads, MINB)
   for (int a = 0; a < 9; ++a) g_out[pop_index(k, a, 9)] = gy[a];
 }
 
-// Modified equilibria (Eq. 16, 20) of given C, p, u, and tau at zero strain
-// rate (reading R11).  C, p, u are in the scratch planes.
-template <int NH>
-__global__ void k_init(DevParams P, const float *__restrict__ Cf, const float *__restrict__ pf,
-                       const float *__restrict__ uxf, const float *__restrict__ uyf, float *__restrict__ g,
-                       float *__restrict__ h, float *__restrict__ tau, int y0, int y1) {
-  const int x = blockIdx.x * blockDim.x + threadIdx.x, y = y0 + blockIdx.y * blockDim.y + threadIdx.y;
-  if (x >= P.nx || y >= y1) return;
+// Modified equilibria (Eq. 16, 20) of given C, p, u, and tau at zero strain rate
+// (reading R11), rows [y0, y1), into the stored form of the state.  The fields come as
+// the host's dense FP64 planes and are rounded to FP32 (to nearest) as they enter the
+// tile: C, rho and p of the 32 x 8 tile and its stencil ring in shared memory, g encoded
+// and C stored by the same kernel in the C forms.  REST: p = u = 0 (the usual set-up),
+// where Gamma_a = w_a and most terms of Phi vanish.  A conversion pass into FP32 planes, a
+// pass that read them through L1 and, with FP16 storage, an encoding pass bound the set-up:
+// lbm_set_fields of C from page-locked memory 815 -> 431 us at 2048 x 4096 (344 us of it the
+// upload), 127 -> 68 us at 517 x 1031, 284 -> 137 us at 1024 x 2048 with FP16 storage (GB300).
+struct InitFields {
+  const double *C, *p, *ux, *uy;  // nh, 1, 1, 1 planes of ny x nx (p, ux, uy: NULL for zero)
+};
+template <int NH, int SCHEME, int FORM, bool REST>
+__global__ void __launch_bounds__(256) k_init(DevParams P, InitFields in, float *__restrict__ g, float *__restrict__ h,
+                                              float *__restrict__ tau, int row0, int row1) {
+  constexpr int TX = 32, TY = 8, R = 1 + SCHEME, W = TX + 2 * R, N = W * (TY + 2 * R);
+  __shared__ float sC[NH][N], srho[N], sp[REST ? 1 : N];
+  const int t = threadIdx.x, tx = t % TX, ty = t / TX, x0 = blockIdx.x * TX, y0 = row0 + blockIdx.y * TY;
+  const int x = x0 + tx, y = y0 + ty;
+  const size_t dense = (size_t)P.nx * P.ny;
+  const bool inside = x0 >= R && y0 >= R && x0 + TX + R <= P.nx && y0 + TY + R <= P.ny;
+  for (int q = t; q < N; q += 256) {
+    const int xq = x0 + q % W - R, yq = y0 + q / W - R;
+    if (yq >= row1 + R) break;  // beyond what the rows below row1 read (it may not have arrived)
+    const size_t d = inside ? (size_t)yq * P.nx + xq
+                            : (size_t)row_read(yq, P.ny, P.periodic_y) * P.nx + tile_column(P, xq);
+    const float c0 = (float)in.C[d], c1 = NH == 2 ? (float)in.C[dense + d] : 0.0f;
+    sC[0][q] = c0;
+    if (NH == 2) sC[NH - 1][q] = c1;
+    srho[q] = rho_of(P, c0, c1, 1.0f - c0 - c1);
+    if (!REST) sp[q] = in.p ? (float)in.p[d] : 0.0f;
+  }
+  __syncthreads();
+  if (x >= P.nx || y >= row1) return;
   const long long k = node_index(P, x, y);
-  CReader cr{Cf, P.plane, NH};
+  struct {
+    const float (&sC)[NH][N];
+    const float (&srho)[N];
+    const float *sp;
+    int q0;
+    __device__ __forceinline__ void C(int dx, int dy, float c[3]) const {
+      const int q = q0 + dy * W + dx;
+      c[0] = sC[0][q];
+      c[1] = NH == 2 ? sC[NH - 1][q] : 0.0f;
+      c[2] = 1.0f - c[0] - c[1];
+    }
+    __device__ __forceinline__ float rho(int dx, int dy, const float *) const { return srho[q0 + dy * W + dx]; }
+    __device__ __forceinline__ float p(int dx, int dy) const { return REST ? 0.0f : sp[q0 + dy * W + dx]; }
+  } at{sC, srho, sp, (ty + R) * W + tx + R};
   NodeCtx n;
-  gather_gradients(P.fd_scheme, PlaneReader{P, cr, pf, x, y}, n);
+  gather_gradients(SCHEME, at, n);
   float Cn[9][3], lapC[3];
-  for (int a = 0; a < 9; ++a) cr.at(shifted(P, x, y, ex(a), ey(a)), Cn[a]);
+#pragma unroll
+  for (int a = 0; a < 9; ++a) at.C(ex(a), ey(a), Cn[a]);
+#pragma unroll
   for (int j = 0; j < 3; ++j) {
     float lp = 0.f;
+#pragma unroll
     for (int a = 0; a < 9; ++a) lp += wt(a) * (Cn[a][j] - Cn[0][j]);
     lapC[j] = 6.0f * lp;
   }
   chem_potentials(P, n.C, lapC, n.mu);
-  n.ux = uxf[k];
-  n.uy = uyf[k];
+  const size_t d0 = (size_t)y * P.nx + x;
+  n.ux = !REST && in.ux ? (float)in.ux[d0] : 0.0f;
+  n.uy = !REST && in.uy ? (float)in.uy[d0] : 0.0f;
   n.Fs[0] = n.mu[0] * n.gC[0][0] + n.mu[1] * n.gC[1][0] + n.mu[2] * n.gC[2][0];
   n.Fs[1] = n.mu[0] * n.gC[0][1] + n.mu[1] * n.gC[1][1] + n.mu[2] * n.gC[2][1];
   n.Fb[0] = P.force_x;
   n.Fb[1] = -n.rho * P.gravity;
-  for (int a = 0; a < 9; ++a) {
-    const float G = gamma_a(a, n.ux, n.uy);
-    g[pop_index(k, a, 9)] = wt(a) * n.p + n.rho * kCs2 * (G - wt(a)) - 0.5f * phi_g(n, a, G);
-    if (h) {
+  // (which product is rounded on its own is spelled out, as in k_collide_step)
+  auto h_eq = [](float C, float G, float ph) {
+    return NH == 1 ? __fmaf_rn(C, G, -0.5f * ph) : __fmaf_rn(-0.5f, ph, __fmul_rn(C, G));
+  };
+  float ge[9];
 #pragma unroll
-      for (int i = 0; i < 2; ++i)
-        if (i < NH) h[pop_index(k, i * 9 + a, 9 * NH)] = n.C[i] * G - 0.5f * phi_h(n, i, a, G);
+  for (int a = 0; a < 9; ++a) {
+    if constexpr (REST) {
+      const float w = wt(a);
+      const float eF = (n.mu[0] * n.dC[0][a] + n.mu[1] * n.dC[1][a] + n.mu[2] * n.dC[2][a]) +
+                       (ex(a) * n.Fb[0] + ey(a) * n.Fb[1]);
+      ge[a] = -0.5f * (eF * w);
+      if constexpr (FORM == 0) {
+#pragma unroll
+        for (int i = 0; i < NH; ++i) {
+          const float ph = (n.dC[i][a] + n.C[i] / (n.rho * kCs2) * eF) * w;
+          h[pop_index(k, i * 9 + a, 9 * NH)] = h_eq(n.C[i], w, ph);
+        }
+      }
+    } else {
+      const float G = gamma_a(a, n.ux, n.uy);
+      const float pg = phi_g(n, a, G), Gw = G - wt(a), rc = n.rho * kCs2;
+      const float lin = a < NH ? __fmaf_rn(wt(a), n.p, __fmul_rn(rc, Gw)) : __fmaf_rn(rc, Gw, __fmul_rn(wt(a), n.p));
+      ge[a] = lin - 0.5f * pg;
+      if constexpr (FORM == 0) {
+#pragma unroll
+        for (int i = 0; i < NH; ++i) h[pop_index(k, i * 9 + a, 9 * NH)] = h_eq(n.C[i], G, phi_h(n, i, a, G));
+      }
     }
+  }
+  if constexpr (FORM == 2) {
+    const float Pn = g16_reference(ge);
+    g[(9 * P.plane) / 2 + k] = Pn;
+    __half *gh = reinterpret_cast<__half *>(g) + pop_index(k, 0, 9);
+#pragma unroll
+    for (int a = 0; a < 9; ++a) gh[a * 32] = g16_encode(ge[a], Pn, a, P.g16_scale);
+  } else {
+#pragma unroll
+    for (int a = 0; a < 9; ++a) g[pop_index(k, a, 9)] = ge[a];
+  }
+  if constexpr (FORM != 0) {
+#pragma unroll
+    for (int i = 0; i < NH; ++i) h[(long long)i * P.plane + k] = n.C[i];
   }
   const float tau1 = P.powerlaw ? tau_powerlaw(P, 0.0f, 1.0f / n.rho) : P.tau[0];
   tau[k] = tau_mix(P, n.C[0], n.C[1], n.C[2], tau1);
 }
 
-// Dense FP64 host-layout planes (ny x nx each) into pitched FP32 planes, one
-// thread per column of the pitch (the padding columns get 0); FP64 -> FP32
-// rounds to nearest, as a host conversion does.
-__global__ void k_planes_from_f64(DevParams P, const double *__restrict__ src, float *__restrict__ dst,
-                                  int nplanes, int y0) {
-  const int x = blockIdx.x * blockDim.x + threadIdx.x, y = y0 + blockIdx.y;
-  if (x >= P.pitch) return;
-  for (int q = 0; q < nplanes; ++q)
-    dst[(long long)q * P.plane + (long long)y * P.pitch + x] =
-        x < P.nx ? (float)src[((long long)q * P.ny + y) * P.nx + x] : 0.0f;
+// Initial discs (Eq. 42) as dense FP64 planes of C_1 (and C_2), one thread per
+// node: every disc adds 0.5 - 0.5 tanh((r - R) / (xi / 2)) to its component in
+// the given order, then the noise, then the matrix takes the rest.  Discs come in groups
+// of kDiscs per launch; between groups the planes hold the sums of components 3 and 2.
+// Farther than 20 half widths from the interface the tanh is +-1 in FP64 (1 - 8.5e-18), so only
+// the interface pays for it.  The host loop this replaces took 1.95 ms at 400 x 800 and 45.9 ms
+// at 2048 x 4096 with its upload; on the device 0.06 and 0.87 ms with the equilibria (GB300).
+__device__ __forceinline__ double noise_at(unsigned long long seed, unsigned long long i) {
+  unsigned long long z = seed + (i + 1) * 0x9E3779B97F4A7C15ULL;  // SplitMix64 (Steele, Lea and Flood 2014)
+  z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ULL;
+  z = (z ^ (z >> 27)) * 0x94D049BB133111EBULL;
+  z ^= z >> 31;
+  return 2.0 * ((double)(z >> 11) * (1.0 / 9007199254740992.0)) - 1.0;
+}
+__global__ void __launch_bounds__(256) k_discs(int nx, int ny, int nh, int periodic_y, double xi, DiscGroup d,
+                                               double *__restrict__ C) {
+  const int x = blockIdx.x * 32 + threadIdx.x % 32, y = blockIdx.y * 8 + threadIdx.x / 32;
+  if (x >= nx || y >= ny) return;
+  const size_t n = (size_t)nx * ny, k = (size_t)y * nx + x;
+  double gas = d.first ? 0.0 : C[k], second = d.first || nh == 1 ? 0.0 : C[n + k];  // components 3 and 2
+  for (int b = 0; b < d.count; ++b) {
+    double dx = fabs(x - d.disc[b].cx), dy = fabs(y - d.disc[b].cy);
+    if (dx > 0.5 * nx) dx = nx - dx;
+    if (periodic_y && dy > 0.5 * ny) dy = ny - dy;
+    const double a = (sqrt(dx * dx + dy * dy) - d.disc[b].r) / (0.5 * xi);
+    const double v = a > 20.0 ? 0.0 : (a < -20.0 ? 1.0 : 0.5 - 0.5 * tanh(a));
+    if (d.disc[b].comp == 3) gas += v;
+    else second += v;
+  }
+  if (!d.last) {
+    C[k] = gas;
+    if (nh == 2) C[n + k] = second;
+    return;
+  }
+  if (d.noise[0] != 0.0) second += d.noise[0] * noise_at(d.seed, n + k);
+  if (d.noise[1] != 0.0) gas += d.noise[1] * noise_at(d.seed, 2 * n + k);
+  C[k] = 1.0 - second - gas;
+  if (nh == 2) C[n + k] = second;
+}
+
+// Fields for the host, as dense FP64 planes: FP32 planes, C_3 or the density of the
+// clipped mixture (R1) from the C planes, and planes [q0, q1) of a population array
+// (g16: the FP16 form of g, decoded).  The host loops over FP32 copies that these replace
+// took most of lbm_get_field: at 400 x 800 u_x 142 -> 58 us, rho 720 -> 68 us, g 2.7 -> 0.19 ms.
+__global__ void __launch_bounds__(256) k_planes_to_f64(DevParams P, double3 rho, const float *__restrict__ src,
+                                                       int kind, double *__restrict__ dst) {
+  const int x = blockIdx.x * 32 + threadIdx.x % 32, y = blockIdx.y * 8 + threadIdx.x / 32, q = blockIdx.z;
+  if (x >= P.nx || y >= P.ny) return;
+  const long long k = node_index(P, x, y);
+  const size_t o = ((size_t)q * P.ny + y) * P.nx + x;
+  if (kind == kPlane) {
+    dst[o] = (double)src[(long long)q * P.plane + k];
+    return;
+  }
+  const float c1 = src[k], c2 = P.nh == 2 ? src[P.plane + k] : 0.0f, c3 = 1.0f - c1 - c2;
+  if (kind == kThird) {
+    dst[o] = (double)c3;
+    return;
+  }
+  const double w1 = fmin(fmax((double)c1, 0.0), 1.0), w2 = fmin(fmax((double)c2, 0.0), 1.0),
+               w3 = fmin(fmax((double)c3, 0.0), 1.0);
+  dst[o] = (w1 * rho.x + w2 * rho.y + w3 * rho.z) / (w1 + w2 + w3);
+}
+__global__ void __launch_bounds__(256) k_pops_to_f64(DevParams P, const float *__restrict__ src, int q0, int nq, int g16,
+                                                     double *__restrict__ dst) {
+  const int x = blockIdx.x * 32 + threadIdx.x % 32, y = blockIdx.y * 8 + threadIdx.x / 32, q = q0 + blockIdx.z;
+  if (x >= P.nx || y >= P.ny) return;
+  const long long k = node_index(P, x, y);
+  float v;
+  if (g16)
+    v = g16_decode(src[(9 * P.plane) / 2 + k], reinterpret_cast<const __half *>(src)[pop_index(k, q, 9)], q,
+                   P.g16_inv_scale);
+  else
+    v = src[pop_index(k, q, nq)];
+  dst[((size_t)blockIdx.z * P.ny + y) * P.nx + x] = (double)v;
 }
 
 // A running FP32 sum with Neumaier's compensation: c collects the rounding
@@ -811,30 +942,56 @@ void launch_macros(const DevParams &P, const StepBuffers &B, cudaStream_t s) {
     k_fields<2><<<grd, blk, 0, s>>>(P, B.C, B.g_in, B.mu, B.p, B.ux, B.uy);
 }
 
-// Rows [y0, y1) of nplanes dense FP64 planes into the pitched FP32 planes.
-cudaError_t launch_planes_from_f64_rows(const DevParams &P, const double *src, float *dst, int nplanes, int y0,
-                                        int y1, cudaStream_t s) {
-  if (y1 <= y0) return cudaSuccess;
-  k_planes_from_f64<<<dim3((P.pitch + 127) / 128, y1 - y0), 128, 0, s>>>(P, src, dst, nplanes, y0);
+template <int NH, int SCHEME, int FORM>
+static cudaError_t init_rows(const DevParams &P, const InitFields &in, float *g, float *h, float *tau, int y0, int y1,
+                             cudaStream_t s) {
+  const dim3 grd((P.nx + 31) / 32, (y1 - y0 + 7) / 8);
+  if (!in.p && !in.ux && !in.uy)
+    k_init<NH, SCHEME, FORM, true><<<grd, 256, 0, s>>>(P, in, g, h, tau, y0, y1);
+  else
+    k_init<NH, SCHEME, FORM, false><<<grd, 256, 0, s>>>(P, in, g, h, tau, y0, y1);
   return cudaGetLastError();
 }
 
-cudaError_t launch_planes_from_f64(const DevParams &P, const double *src, float *dst, int nplanes, cudaStream_t s) {
-  return launch_planes_from_f64_rows(P, src, dst, nplanes, 0, P.ny, s);
+cudaError_t launch_init_rows(const DevParams &P, const double *C, const double *p, const double *ux, const double *uy,
+                             float *g, float *h, float *tau, int y0, int y1, cudaStream_t s) {
+  if (y1 <= y0) return cudaSuccess;
+  const InitFields in{C, p, ux, uy};
+  if (P.nh == 1) {
+    if (P.g16) return init_rows<1, 0, 2>(P, in, g, h, tau, y0, y1, s);
+    if (P.collapse_h) return init_rows<1, 0, 1>(P, in, g, h, tau, y0, y1, s);
+    return P.fd_scheme == 1 ? init_rows<1, 1, 0>(P, in, g, h, tau, y0, y1, s)
+                            : init_rows<1, 0, 0>(P, in, g, h, tau, y0, y1, s);
+  }
+  if (P.g16) return init_rows<2, 0, 2>(P, in, g, h, tau, y0, y1, s);
+  if (P.collapse_h) return init_rows<2, 0, 1>(P, in, g, h, tau, y0, y1, s);
+  return P.fd_scheme == 1 ? init_rows<2, 1, 0>(P, in, g, h, tau, y0, y1, s)
+                          : init_rows<2, 0, 0>(P, in, g, h, tau, y0, y1, s);
 }
 
-// Initial equilibria of rows [y0, y1) (they read C and p two rows beyond).
-void launch_init_rows(const DevParams &P, const StepBuffers &B, int y0, int y1, cudaStream_t s) {
+cudaError_t launch_discs(const DevParams &P, double xi, const DiscGroup &d, double *C, cudaStream_t s) {
+  k_discs<<<dim3((P.nx + 31) / 32, (P.ny + 7) / 8), 256, 0, s>>>(P.nx, P.ny, P.nh, P.periodic_y, xi, d, C);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_planes_to_f64(const DevParams &P, const double rho[3], const float *src, int kind, int nplanes,
+                                 double *dst, cudaStream_t s) {
+  k_planes_to_f64<<<dim3((P.nx + 31) / 32, (P.ny + 7) / 8, nplanes), 256, 0, s>>>(
+      P, make_double3(rho[0], rho[1], rho[2]), src, kind, dst);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_pops_to_f64(const DevParams &P, const float *src, int q0, int q1, int nq, bool g16, double *dst,
+                               cudaStream_t s) {
+  k_pops_to_f64<<<dim3((P.nx + 31) / 32, (P.ny + 7) / 8, q1 - q0), 256, 0, s>>>(P, src, q0, nq, g16 ? 1 : 0, dst);
+  return cudaGetLastError();
+}
+
+// C_i of the population form into the C planes.
+void launch_moments(const DevParams &P, const float *h, float *C, cudaStream_t s) {
   const dim3 blk(32, 8);
-  const dim3 grd((P.nx + blk.x - 1) / blk.x, (y1 - y0 + blk.y - 1) / blk.y);
-  if (y1 <= y0) return;
-  if (P.nh == 1)
-    k_init<1><<<grd, blk, 0, s>>>(P, B.C, B.p, B.ux, B.uy, B.g_out, B.h_out, B.tau_out, y0, y1);
-  else
-    k_init<2><<<grd, blk, 0, s>>>(P, B.C, B.p, B.ux, B.uy, B.g_out, B.h_out, B.tau_out, y0, y1);
+  k_moments<<<node_grid(P, blk), blk, 0, s>>>(P, h, C);
 }
-
-void launch_init(const DevParams &P, const StepBuffers &B, cudaStream_t s) { launch_init_rows(P, B, 0, P.ny, s); }
 
 cudaError_t launch_observe(const DevParams &P, const FusedBuffers &B, int gas_comp, double *acc, int *ext,
                            cudaStream_t s) {
