@@ -52,16 +52,16 @@ struct lbm_batch {
   bool persistent = false;
   long long spin_limit = kDefaultSpinLimit;
   cudaGraphExec_t pgraph = nullptr;  // one persistent launch of kPersistSteps steps
-  int pgraph_nwork = -1, pgraph_variant = -1;
+  int pgraph_nwork = -1, pgraph_variant = -1, pgraph_grid = -1;
   long long pgraph_limit = -1;
   size_t work_cap = 0;
-  int nwork = 0;
+  int nwork = 0, grid = 0;  // items of the list; CTAs that share it (0: one per item, or a counter)
   int variant = 0;
   int nh = 1;
   int form = 0;  // 0 populations, 1 C state (collapse_h), 2 FP16 g and C (storage 1)
   bool work_valid = false;
   cudaGraphExec_t graph = nullptr;
-  int graph_nwork = -1, graph_variant = -1;
+  int graph_nwork = -1, graph_variant = -1, graph_grid = -1;
   std::string last_error;
 
   lbm_status fail(lbm_status s, const std::string &m) {
@@ -78,35 +78,108 @@ struct lbm_batch {
     for (auto *x : h) delete x;
   }
 
-  // Work list of the active, initialised cases for configuration v (tiles, or
-  // strips x row segments of a sweep); uploads it.
-  cudaError_t build_work(int v, int *count) {
-    std::vector<lbm::WorkItem> w;
-    for (int i = 0; i < n; ++i) {
-      if (!active[i] || !h[i]->initialized) continue;
-      int tx = 32, ty = 8;
-      lbm::batched_variant_tile(nh, v, &tx, &ty);
-      const int ny = h[i]->dp.ny;
-      if (lbm::batched_variant_is_sweep(nh, v)) {
-        // sweep segments: the rows of a strip split evenly (an even number of
-        // rows each, as the two-row pipeline steps take them), so that no
-        // short last segment pays a whole pipeline fill for a few rows
-        const int nseg = (ny + ty - 1) / ty;
-        int len = (ny + nseg - 1) / nseg;
-        len += len & 1;
-        for (int y0 = 0; y0 < ny; y0 += len)
-          for (int x0 = 0; x0 < h[i]->dp.nx; x0 += tx) w.push_back({i, x0, y0, y0 + len < ny ? y0 + len : ny});
-      } else {
-        for (int y0 = 0; y0 < ny; y0 += ty)
-          for (int x0 = 0; x0 < h[i]->dp.nx; x0 += tx) w.push_back({i, x0, y0, y0 + ty < ny ? y0 + ty : ny});
-      }
+  // Shared lists of a sweep: the strips of every running case laid end to end and cut
+  // into one share per CTA slot, shares equal in rows plus the pipeline fill of each
+  // piece (the smallest such size for which the slots suffice, by bisection).  A piece has
+  // at least kLeast rows and starts at a multiple of rs of its strip.  Piece k of share b stands at
+  // k * shares + b, empty pieces (y0 = y1) where a share has fewer.  Returns the shares, 0 if
+  // the padded list does not fit in cap.
+  static int share_out(const std::vector<lbm::WorkItem> &strips, int rs, int slots, size_t cap,
+                       std::vector<lbm::WorkItem> *out) {
+    constexpr int kLeast = 8;
+    const int fill = 3 * rs + rs * ((6 + rs - 1) / rs);
+    long long rows = 0;
+    int longest = 0;
+    for (const auto &s : strips) {
+      rows += s.y1;
+      longest = std::max(longest, s.y1);
     }
-    // longest items first: the CTAs take items in order (one launch per step,
-    // or from a counter in the persistent launch), which then approximates the
-    // longest-processing-time schedule
-    std::stable_sort(w.begin(), w.end(), [](const lbm::WorkItem &a, const lbm::WorkItem &b) {
-      return a.y1 - a.y0 > b.y1 - b.y0;
-    });
+    // pieces of each share of `size` rows with their fills
+    auto cut = [&](long long size, std::vector<std::vector<lbm::WorkItem>> *shares) {
+      int used = 0;
+      long long left = 0;  // of the current share
+      for (const auto &s : strips) {
+        int y = 0;
+        while (y < s.y1) {
+          if (used == 0 || left - fill < std::min(kLeast, s.y1 - y)) {
+            ++used;
+            left = size;
+            if (shares) shares->emplace_back();
+          }
+          int len = (int)std::min<long long>(s.y1 - y, std::max<long long>(left - fill, kLeast));
+          if (len < s.y1 - y) len -= len % rs;
+          if (s.y1 - y - len < kLeast) len = s.y1 - y;  // no crumb for the next share
+          if (shares) shares->back().push_back({s.case_id, s.x0, y, y + len});
+          y += len;
+          left -= len + fill;
+        }
+      }
+      return used;
+    };
+    long long lo = 1, hi = rows + (long long)fill * (long long)strips.size() + fill + kLeast;  // hi: one share
+    while (lo < hi) {
+      const long long mid = (lo + hi) / 2;
+      if (cut(mid, nullptr) <= slots) hi = mid;
+      else lo = mid + 1;
+    }
+    std::vector<std::vector<lbm::WorkItem>> shares;
+    const int n = cut(hi, &shares);
+    size_t deepest = 0;
+    for (const auto &s : shares) deepest = std::max(deepest, s.size());
+    if (n > slots || deepest * (size_t)n > cap) return 0;
+    out->assign(deepest * (size_t)n, lbm::WorkItem{0, 0, 0, 0});
+    for (int b = 0; b < n; ++b)
+      for (size_t k = 0; k < shares[b].size(); ++k) (*out)[k * (size_t)n + b] = shares[b][k];
+    return n;
+  }
+
+  // Work list of the active, initialised cases for configuration v (tiles, strips x
+  // row segments, or shared lists of a sweep); uploads it.  *ctas: the CTAs that share
+  // it, 0 for one item per CTA.
+  cudaError_t build_work(int v, int *count, int *ctas) {
+    std::vector<lbm::WorkItem> w;
+    int tx = 32, ty = 8;
+    constexpr int rs = 2;  // rows per pipeline step of every batched sweep
+    lbm::batched_variant_tile(nh, v, &tx, &ty);
+    *ctas = 0;
+    const bool sweep = lbm::batched_variant_is_sweep(nh, v);
+    if (sweep && ty == 0) {
+      std::vector<lbm::WorkItem> strips;  // whole strips: y0 = 0, y1 = rows
+      for (int i = 0; i < n; ++i) {
+        if (!active[i] || !h[i]->initialized) continue;
+        for (int x0 = 0; x0 < h[i]->dp.nx; x0 += tx) strips.push_back({i, x0, 0, h[i]->dp.ny});
+      }
+      int slots = 0;
+      const cudaError_t e = lbm::sweep_batched_slots(nh, form, v, persistent, &slots);
+      if (e != cudaSuccess) return e;
+      if (!strips.empty()) *ctas = share_out(strips, rs, slots, work_cap, &w);
+      if (*ctas == 0) ty = 96;  // no room for the lists: segments
+    }
+    if (*ctas == 0) {
+      for (int i = 0; i < n; ++i) {
+        if (!active[i] || !h[i]->initialized) continue;
+        const int ny = h[i]->dp.ny;
+        if (sweep) {
+          // sweep segments: the rows of a strip split evenly (a multiple of the rows of a
+          // pipeline step each), so that no short last segment pays a whole pipeline
+          // fill for a few rows
+          const int nseg = (ny + ty - 1) / ty;
+          int len = (ny + nseg - 1) / nseg;
+          len = (len + rs - 1) / rs * rs;
+          for (int y0 = 0; y0 < ny; y0 += len)
+            for (int x0 = 0; x0 < h[i]->dp.nx; x0 += tx) w.push_back({i, x0, y0, y0 + len < ny ? y0 + len : ny});
+        } else {
+          for (int y0 = 0; y0 < ny; y0 += ty)
+            for (int x0 = 0; x0 < h[i]->dp.nx; x0 += tx) w.push_back({i, x0, y0, y0 + ty < ny ? y0 + ty : ny});
+        }
+      }
+      // longest items first: the CTAs take items in order (one launch per step,
+      // or from a counter in the persistent launch), which then approximates the
+      // longest-processing-time schedule
+      std::stable_sort(w.begin(), w.end(), [](const lbm::WorkItem &a, const lbm::WorkItem &b) {
+        return a.y1 - a.y0 > b.y1 - b.y0;
+      });
+    }
     if (w.size() > work_cap) return cudaErrorInvalidValue;  // the arena's work list is sized for 32 x 8 items
     *count = (int)w.size();
     if (w.empty()) return cudaSuccess;
@@ -144,16 +217,16 @@ static lbm_status persistent_steps(lbm_batch *b, long long nsteps) {
   auto one_launch = [&](int steps) {
     cudaError_t r = cudaMemsetAsync(b->d_sync, 0, sizeof(lbm::GridSync), b->stream);
     if (r == cudaSuccess)
-      r = lbm::launch_sweep_persistent(b->nh, b->form, b->d_cases, b->d_work, b->nwork, 0, steps, b->d_sync,
+      r = lbm::launch_sweep_persistent(b->nh, b->form, b->d_cases, b->d_work, b->nwork, b->grid, 0, steps, b->d_sync,
                                        b->spin_limit, b->stream, b->variant, &grid);
     return r;
   };
   const bool capturable = b->stream != nullptr && b->stream != cudaStreamLegacy && b->stream != cudaStreamPerThread;
   const long long full = capturable ? nsteps / kPersistSteps : 0;
   if (full > 0 && (!b->pgraph || b->pgraph_nwork != b->nwork || b->pgraph_variant != b->variant ||
-                   b->pgraph_limit != b->spin_limit)) {
+                   b->pgraph_grid != b->grid || b->pgraph_limit != b->spin_limit)) {
     // kernel attributes and occupancy are queried outside the capture
-    e = lbm::launch_sweep_persistent(b->nh, b->form, b->d_cases, b->d_work, b->nwork, 0, 0, b->d_sync,
+    e = lbm::launch_sweep_persistent(b->nh, b->form, b->d_cases, b->d_work, b->nwork, b->grid, 0, 0, b->d_sync,
                                      b->spin_limit, b->stream, b->variant, &grid);
     if (e != cudaSuccess) return b->cuda_fail(e, "lbm_batch_step persistent prepare");
     if (b->pgraph) cudaGraphExecDestroy(b->pgraph);
@@ -168,6 +241,7 @@ static lbm_status persistent_steps(lbm_batch *b, long long nsteps) {
     if (e != cudaSuccess) return b->cuda_fail(e, "lbm_batch_step persistent graph capture");
     b->pgraph_nwork = b->nwork;
     b->pgraph_variant = b->variant;
+    b->pgraph_grid = b->grid;
     b->pgraph_limit = b->spin_limit;
   }
   std::vector<unsigned> err(b->n);
@@ -300,14 +374,15 @@ lbm_status lbm_batch_autotune(lbm_batch *b, int reps, int *chosen) {
   int best = 0;
   float best_ms = 0.f;
   for (int v = 0; v < nv && e == cudaSuccess; ++v) {
-    int nw = 0;
-    e = b->build_work(v, &nw);
+    int nw = 0, grid = 0;
+    e = b->build_work(v, &nw, &grid);
     if (e != cudaSuccess || nw == 0) break;
     // parity 0 reads every case's current state and writes its spare buffers
-    e = lbm::launch_batched_step(b->nh, b->form, b->d_cases, b->d_work, nw, 0, b->stream, v);
+    e = lbm::launch_batched_step(b->nh, b->form, b->d_cases, b->d_work, nw, grid, 0, b->stream, v);
     if (e != cudaSuccess) break;
     cudaEventRecord(e0, b->stream);
-    for (int r = 0; r < reps; ++r) lbm::launch_batched_step(b->nh, b->form, b->d_cases, b->d_work, nw, 0, b->stream, v);
+    for (int r = 0; r < reps; ++r)
+      lbm::launch_batched_step(b->nh, b->form, b->d_cases, b->d_work, nw, grid, 0, b->stream, v);
     cudaEventRecord(e1, b->stream);
     e = cudaEventSynchronize(e1);
     float ms = 0.f;
@@ -331,7 +406,7 @@ lbm_status lbm_batch_step(lbm_batch *b, long long nsteps) {
   if (nsteps == 0) return LBM_OK;
   cudaError_t e = cudaSuccess;
   if (!b->work_valid) {
-    e = b->build_work(b->variant, &b->nwork);
+    e = b->build_work(b->variant, &b->nwork, &b->grid);
     if (e != cudaSuccess) return b->cuda_fail(e, "lbm_batch_step work list");
     b->work_valid = true;
   }
@@ -343,16 +418,18 @@ lbm_status lbm_batch_step(lbm_batch *b, long long nsteps) {
   // graphs need a capturable stream: not the legacy or per-thread default stream
   const bool capturable = b->stream != nullptr && b->stream != cudaStreamLegacy && b->stream != cudaStreamPerThread;
   const long long graphs = capturable ? nsteps / kGraphSteps : 0;
-  if (graphs > 0 && (!b->graph || b->graph_nwork != b->nwork || b->graph_variant != b->variant)) {
+  if (graphs > 0 && (!b->graph || b->graph_nwork != b->nwork || b->graph_variant != b->variant ||
+                     b->graph_grid != b->grid)) {
     // kernel attributes are set outside the capture
-    e = lbm::launch_batched_step(b->nh, b->form, b->d_cases, b->d_work, 0, 0, b->stream, b->variant);
+    e = lbm::launch_batched_step(b->nh, b->form, b->d_cases, b->d_work, 0, 0, 0, b->stream, b->variant);
     if (e != cudaSuccess) return b->cuda_fail(e, "lbm_batch_step prepare");
     if (b->graph) cudaGraphExecDestroy(b->graph);
     b->graph = nullptr;
     cudaGraph_t g = nullptr;
     e = cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal);
     for (int t = 0; t < kGraphSteps && e == cudaSuccess; ++t)
-      e = lbm::launch_batched_step(b->nh, b->form, b->d_cases, b->d_work, b->nwork, t & 1, b->stream, b->variant);
+      e = lbm::launch_batched_step(b->nh, b->form, b->d_cases, b->d_work, b->nwork, b->grid, t & 1, b->stream,
+                                   b->variant);
     cudaError_t ec = cudaStreamEndCapture(b->stream, &g);
     if (e == cudaSuccess) e = ec;
     if (e == cudaSuccess) e = cudaGraphInstantiate(&b->graph, g, 0);
@@ -360,10 +437,11 @@ lbm_status lbm_batch_step(lbm_batch *b, long long nsteps) {
     if (e != cudaSuccess) return b->cuda_fail(e, "lbm_batch_step graph capture");
     b->graph_nwork = b->nwork;
     b->graph_variant = b->variant;
+    b->graph_grid = b->grid;
   }
   for (long long r = 0; r < graphs && e == cudaSuccess; ++r) e = cudaGraphLaunch(b->graph, b->stream);
   for (long long t = graphs * kGraphSteps; t < nsteps && e == cudaSuccess; ++t)
-    e = lbm::launch_batched_step(b->nh, b->form, b->d_cases, b->d_work, b->nwork, (int)(t & 1), b->stream,
+    e = lbm::launch_batched_step(b->nh, b->form, b->d_cases, b->d_work, b->nwork, b->grid, (int)(t & 1), b->stream,
                                  b->variant);
   if (e != cudaSuccess) return b->cuda_fail(e, "lbm_batch_step launch");
   std::vector<unsigned> err(b->n);

@@ -67,22 +67,28 @@ bool fused_supported(const DevParams &P);
 // segment)) first, then tiles (work items (case, tile)).
 int batched_variant_count(int nh);
 bool batched_variant_is_sweep(int nh, int v);
+// Tile of configuration v, or strip width and segment rows (0: shared lists).
 void batched_variant_tile(int nh, int v, int *tx, int *ty);
 int sweep_batched_count(int nh);
+// rs (may be null): rows per pipeline step
 void sweep_batched_shape(int nh, int v, int *tx, int *rows);
-// form: 0 populations g, h; 1 g and C (collapse_h); 2 FP16 g deviations and C
-cudaError_t launch_sweep_batched(int nh, int form, const BatchCase *cases, const WorkItem *work, int nwork,
+// CTAs of configuration v that the device holds at once.
+cudaError_t sweep_batched_slots(int nh, int form, int v, bool persistent, int *ctas);
+// form: 0 populations g, h; 1 g and C (collapse_h); 2 FP16 g deviations and C.
+// grid: CTAs that share the list out as items b, b + grid, ... (0: one CTA per item).
+cudaError_t launch_sweep_batched(int nh, int form, const BatchCase *cases, const WorkItem *work, int nwork, int grid,
                                  int parity, cudaStream_t s, int v);
-cudaError_t launch_batched_step(int nh, int form, const BatchCase *cases, const WorkItem *work, int nwork,
+cudaError_t launch_batched_step(int nh, int form, const BatchCase *cases, const WorkItem *work, int nwork, int grid,
                                 int parity, cudaStream_t s, int v);
 // nsteps time steps of every work item in one persistent cooperative launch
 // (sweep configurations v < sweep_batched_count(nh) only): the CTAs that fit
 // on the device at once share the items of a step and meet at a grid barrier
 // between steps; a barrier wait gives up after spin_limit polls, sets
-// kSyncTimeout in sync->status and the kernel returns.  *grid = CTAs launched.
-cudaError_t launch_sweep_persistent(int nh, int form, const BatchCase *cases, const WorkItem *work, int nwork,
+// kSyncTimeout in sync->status and the kernel returns.  grid as above, at most the
+// CTAs that fit (0: items from a counter, all CTAs that fit); *launched = CTAs launched.
+cudaError_t launch_sweep_persistent(int nh, int form, const BatchCase *cases, const WorkItem *work, int nwork, int grid,
                                     int parity0, int nsteps, GridSync *sync, long long spin_limit, cudaStream_t s,
-                                    int v, int *grid);
+                                    int v, int *launched);
 // Launch configurations of the fused step: row sweeps (strip width, rows per
 // pipeline step, threads, CTAs per SM), then tiles (tile, threads, CTAs per SM).
 int sweep_variant_count(const DevParams &P);

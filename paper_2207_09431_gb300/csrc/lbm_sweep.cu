@@ -475,23 +475,28 @@ __global__ void __launch_bounds__(NT, MINB) k_step_sweep(DevParams P, FusedBuffe
                                         *reinterpret_cast<PipeSmem<TX, RS, NH, FORM != 0> *>(smem_raw));
 }
 
-// Many lattices in one launch: CTA b sweeps work item b = (case, strip origin,
-// rows [y0, y1)); the case's parameters and buffers are staged in shared memory.
-// parity selects which of the case's two buffer sets is the input this step.
+// Many lattices in one launch: CTA b sweeps the work items b, b + G, ... of the
+// list, an item being (case, strip origin, rows [y0, y1)) and empty where y1 <= y0; the
+// case's parameters and buffers are staged in shared memory.  parity selects which
+// of the case's two buffer sets is the input this step.
 template <int TX, int RS, int NH, int FORM, int NT, int MINB>
 __global__ void __launch_bounds__(NT, MINB) k_sweep_batched(const BatchCase *__restrict__ cases,
-                                                            const WorkItem *__restrict__ work, int parity) {
+                                                            const WorkItem *__restrict__ work, int nwork, int parity) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ DevParams sP;
   __shared__ FusedBuffers sB;
-  const WorkItem w = work[blockIdx.x];
-  if (threadIdx.x == 0) {
-    sP = cases[w.case_id].P;
-    sB = cases[w.case_id].B[cases[w.case_id].base_parity ^ parity];
+  for (int i = blockIdx.x; i < nwork; i += gridDim.x) {
+    const WorkItem w = work[i];
+    if (w.y1 <= w.y0) continue;
+    if (i != blockIdx.x) __syncthreads();  // sP and sB are in use until the item before is done
+    if (threadIdx.x == 0) {
+      sP = cases[w.case_id].P;
+      sB = cases[w.case_id].B[cases[w.case_id].base_parity ^ parity];
+    }
+    __syncthreads();
+    sweep_body<TX, RS, NH, FORM, 2, NT>(sP, sB, w.x0, w.y0, w.y1,
+                                        *reinterpret_cast<PipeSmem<TX, RS, NH, FORM != 0> *>(smem_raw));
   }
-  __syncthreads();
-  sweep_body<TX, RS, NH, FORM, 2, NT>(sP, sB, w.x0, w.y0, w.y1,
-                                      *reinterpret_cast<PipeSmem<TX, RS, NH, FORM != 0> *>(smem_raw));
 }
 
 // Grid-wide barrier between the time steps of the persistent batched sweep.
@@ -545,10 +550,11 @@ __device__ __forceinline__ bool grid_barrier(GridSync *gs, unsigned nblocks, lon
 // what this one wrote.  Every CTA takes items until the counter runs past the
 // list, before it reaches the barrier, so a step's counter is idle from that
 // barrier on: block 0 clears it during the step after, for the step after that.
+// With fixed lists (work shared out beforehand) CTA b takes items b, b + G, ... instead.
 template <int TX, int RS, int NH, int FORM, int NT, int MINB>
 __global__ void __launch_bounds__(NT, MINB) k_sweep_persistent(const BatchCase *__restrict__ cases,
                                                                const WorkItem *__restrict__ work, int nwork,
-                                                               int parity0, int nsteps, GridSync *sync,
+                                                               int fixed, int parity0, int nsteps, GridSync *sync,
                                                                long long spin_limit) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ DevParams sP;
@@ -559,6 +565,10 @@ __global__ void __launch_bounds__(NT, MINB) k_sweep_persistent(const BatchCase *
     if (blockIdx.x == 0 && threadIdx.x == 0) sync->next[(t + 1) & 1] = 0u;  // last used in step t - 1
     for (int i = blockIdx.x; i < nwork;) {
       const WorkItem w = work[i];
+      if (w.y1 <= w.y0) {  // fixed lists only: the rest of this CTA's share is empty
+        i += gridDim.x;
+        continue;
+      }
       if (threadIdx.x == 0) {
         sP = cases[w.case_id].P;
         sB = cases[w.case_id].B[cases[w.case_id].base_parity ^ parity];
@@ -567,6 +577,10 @@ __global__ void __launch_bounds__(NT, MINB) k_sweep_persistent(const BatchCase *
       sweep_body<TX, RS, NH, FORM, 2, NT>(sP, sB, w.x0, w.y0, w.y1,
                                           *reinterpret_cast<PipeSmem<TX, RS, NH, FORM != 0> *>(smem_raw));
       __syncthreads();  // sP and sB are rewritten by the next item
+      if (fixed) {
+        i += gridDim.x;
+        continue;
+      }
       if (threadIdx.x == 0) s_next = (int)gridDim.x + (int)atomicAdd(&sync->next[t & 1], 1u);
       __syncthreads();
       i = s_next;
@@ -697,132 +711,135 @@ static cudaError_t sweep_dispatch(int v, const DevParams &P, const FusedBuffers 
   }
 }
 
-// Batched sweeps (work items of the strip width and segment length of the
-// configuration; segments of 48 or 96 rows keep thousands of items for an
-// ensemble of small lattices).
+// One shape of the batched sweep: its kernels, and the CTAs of each that the device
+// holds at once (looked up on first use, outside any stream capture).
 template <int TX, int RS, int NH, int FORM, int NT, int MINB>
-static cudaError_t launch_sweep_batched_t(const BatchCase *cases, const WorkItem *work, int nwork, int parity,
-                                          cudaStream_t st) {
-  const size_t smem = sizeof(PipeSmem<TX, RS, NH, FORM != 0>);
-  static bool configured = false;
-  if (!configured) {
-    cudaError_t e = cudaFuncSetAttribute(k_sweep_batched<TX, RS, NH, FORM, NT, MINB>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    configured = true;
-  }
-  if (nwork <= 0) return cudaSuccess;
-  k_sweep_batched<TX, RS, NH, FORM, NT, MINB><<<nwork, NT, smem, st>>>(cases, work, parity);
-  return cudaGetLastError();
-}
-
-template <int TX, int RS, int NH, int FORM, int NT, int MINB>
-static cudaError_t launch_sweep_persistent_t(const BatchCase *cases, const WorkItem *work, int nwork, int parity0,
-                                             int nsteps, GridSync *sync, long long spin_limit, cudaStream_t st,
-                                             int *grid) {
-  auto kern = k_sweep_persistent<TX, RS, NH, FORM, NT, MINB>;
-  const size_t smem = sizeof(PipeSmem<TX, RS, NH, FORM != 0>);
-  static int resident = 0;
-  if (!resident) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+struct BatchedSweep {
+  static constexpr size_t kSmem = sizeof(PipeSmem<TX, RS, NH, FORM != 0>);
+  template <typename K>
+  static cudaError_t resident(K kernel, int *ctas) {
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem);
     int dev = 0, sms = 0, per_sm = 0;
     if (e == cudaSuccess) e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, NT, smem);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, NT, kSmem);
+    if (e == cudaSuccess && per_sm < 1) e = cudaErrorInvalidConfiguration;
+    if (e == cudaSuccess) *ctas = per_sm * sms;
+    return e;
+  }
+  static cudaError_t slots(bool persistent, int *ctas) {
+    static int of_step = 0, of_persistent = 0;
+    int &n = persistent ? of_persistent : of_step;
+    if (!n) {
+      const cudaError_t e = persistent ? resident(k_sweep_persistent<TX, RS, NH, FORM, NT, MINB>, &n)
+                                       : resident(k_sweep_batched<TX, RS, NH, FORM, NT, MINB>, &n);
+      if (e != cudaSuccess) {
+        n = 0;
+        return e;
+      }
+    }
+    *ctas = n;
+    return cudaSuccess;
+  }
+  static cudaError_t step(const BatchCase *cases, const WorkItem *work, int nwork, int grid, int parity,
+                          cudaStream_t st) {
+    int ctas = 0;
+    const cudaError_t e = slots(false, &ctas);
+    if (e != cudaSuccess || nwork <= 0) return e;
+    k_sweep_batched<TX, RS, NH, FORM, NT, MINB><<<grid > 0 ? grid : nwork, NT, kSmem, st>>>(cases, work, nwork, parity);
+    return cudaGetLastError();
+  }
+  static cudaError_t persistent(const BatchCase *cases, const WorkItem *work, int nwork, int grid, int parity0,
+                                int nsteps, GridSync *sync, long long spin_limit, cudaStream_t st, int *launched) {
+    int ctas = 0;
+    const cudaError_t e = slots(true, &ctas);
     if (e != cudaSuccess) return e;
-    if (per_sm < 1) return cudaErrorInvalidConfiguration;
-    resident = per_sm * sms;
+    if (grid > ctas) return cudaErrorInvalidConfiguration;  // the CTAs wait for one another: all must be resident
+    const int nb = grid > 0 ? grid : (nwork < ctas ? nwork : ctas);
+    if (launched) *launched = nb;
+    if (nwork <= 0 || nsteps <= 0) return cudaSuccess;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(nb);
+    cfg.blockDim = dim3(NT);
+    cfg.dynamicSmemBytes = kSmem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeCooperative;
+    attr[0].val.cooperative = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, k_sweep_persistent<TX, RS, NH, FORM, NT, MINB>, cases, work, nwork,
+                              grid > 0 ? 1 : 0, parity0, nsteps, sync, spin_limit);
   }
-  const int nb = nwork < resident ? nwork : resident;
-  if (grid) *grid = nb;
-  if (nwork <= 0 || nsteps <= 0) return cudaSuccess;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(nb);
-  cfg.blockDim = dim3(NT);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeCooperative;
-  attr[0].val.cooperative = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kern, cases, work, nwork, parity0, nsteps, sync, spin_limit);
-}
+};
 
-template <int NH, int FORM>
-static cudaError_t sweep_persistent_dispatch(int v, const BatchCase *c, const WorkItem *w, int n, int parity0,
-                                             int nsteps, GridSync *sync, long long lim, cudaStream_t s, int *grid) {
-  if constexpr (NH == 1) {
-    switch (v) {
-      case 2:
-      case 6:
-      case 7:
-      case 8: return launch_sweep_persistent_t<60, 2, NH, FORM, 160, 3>(c, w, n, parity0, nsteps, sync, lim, s, grid);
-      case 3: return launch_sweep_persistent_t<64, 2, NH, FORM, 160, 3>(c, w, n, parity0, nsteps, sync, lim, s, grid);
-      default: return launch_sweep_persistent_t<58, 2, NH, FORM, 128, 3>(c, w, n, parity0, nsteps, sync, lim, s, grid);
-    }
-  } else {
-    if (v == 1) return launch_sweep_persistent_t<62, 2, NH, FORM, 160, 2>(c, w, n, parity0, nsteps, sync, lim, s, grid);
-    return launch_sweep_persistent_t<64, 2, NH, FORM, 160, 2>(c, w, n, parity0, nsteps, sync, lim, s, grid);
-  }
-}
+// Batched configurations: strip width (two rows per pipeline step) and either the rows of a
+// segment (one item per CTA; in the persistent launch from a counter) or 0 for shared
+// lists: the strips of all cases laid end to end and cut into one share per CTA slot.
+// Short segments give many items for the waves, long ones fewer pipeline fills per item;
+// the shares fill the device once with the least fill.  The autotuner picks; measured
+// on a GB300, best segments against best shares: 256 cases of 100 x 200 281 against 230 us per
+// step (100-column strips, which fit the lattice: 58- and 60-column strips leave a sixth of
+// their columns empty there), in the C form 291 against 269 us (60 columns; the larger record
+// of that form leaves one CTA of the 100-column strips per SM); 48 cases of 100 x 200 to 300 x
+// 600 196 against 187 us, C form 204 against 194 us.  Shares of 58 columns were no better than
+// those of 60, nor four-row strips of 50.
+static const int kShapes1[12][2] = {{58, 48}, {58, 96},  {60, 48},  {64, 48},  {58, 64}, {58, 72},
+                                    {60, 64}, {60, 128}, {60, 200}, {58, 160}, {60, 0},  {100, 0}};
+static const int kShapes2[4][2] = {{64, 48}, {62, 48}, {64, 0}, {62, 0}};
 
-int sweep_batched_count(int nh) { return nh == 1 ? 10 : 2; }
+int sweep_batched_count(int nh) { return nh == 1 ? 12 : 4; }
 
-// (strip width, segment rows): short segments give many work items for the
-// waves, long ones fewer pipeline fill steps per item
 void sweep_batched_shape(int nh, int v, int *tx, int *rows) {
-  static const int s1[10][2] = {{58, 48}, {58, 96}, {60, 48}, {64, 48}, {58, 64}, {58, 72}, {60, 64},
-                                {60, 128}, {60, 200}, {58, 160}};
-  static const int s2[2][2] = {{64, 48}, {62, 48}};
   if (v < 0 || v >= sweep_batched_count(nh)) v = 0;
-  *tx = nh == 1 ? s1[v][0] : s2[v][0];
-  *rows = nh == 1 ? s1[v][1] : s2[v][1];
+  *tx = nh == 1 ? kShapes1[v][0] : kShapes2[v][0];
+  *rows = nh == 1 ? kShapes1[v][1] : kShapes2[v][1];
 }
 
-template <int NH, int FORM>
-static cudaError_t sweep_batched_dispatch(int v, const BatchCase *c, const WorkItem *w, int n, int parity,
-                                          cudaStream_t s) {
+// Calls f with the kernels of configuration v.
+template <int NH, int FORM, typename F>
+static cudaError_t with_shape(int v, F &&f) {
   if constexpr (NH == 1) {
-    switch (v) {
-      case 2:
-      case 6:
-      case 7:
-      case 8: return launch_sweep_batched_t<60, 2, NH, FORM, 160, 3>(c, w, n, parity, s);
-      case 3: return launch_sweep_batched_t<64, 2, NH, FORM, 160, 3>(c, w, n, parity, s);
-      default: return launch_sweep_batched_t<58, 2, NH, FORM, 128, 3>(c, w, n, parity, s);
+    switch (kShapes1[v][0]) {
+      case 60: return f(BatchedSweep<60, 2, NH, FORM, 160, 3>());
+      case 64: return f(BatchedSweep<64, 2, NH, FORM, 160, 3>());
+      case 100: return f(BatchedSweep<100, 2, NH, FORM, 224, 2>());
+      default: return f(BatchedSweep<58, 2, NH, FORM, 128, 3>());
     }
   } else {
-    if (v == 1) return launch_sweep_batched_t<62, 2, NH, FORM, 160, 2>(c, w, n, parity, s);
-    return launch_sweep_batched_t<64, 2, NH, FORM, 160, 2>(c, w, n, parity, s);
+    if (kShapes2[v][0] == 62) return f(BatchedSweep<62, 2, NH, FORM, 160, 2>());
+    return f(BatchedSweep<64, 2, NH, FORM, 160, 2>());
   }
 }
-
-cudaError_t launch_sweep_batched(int nh, int form, const BatchCase *cases, const WorkItem *work, int nwork,
-                                 int parity, cudaStream_t s, int v) {
+template <typename F>
+static cudaError_t with_sweep(int nh, int form, int v, F &&f) {
   if (v < 0 || v >= sweep_batched_count(nh)) v = 0;
   if (nh == 1) {
-    if (form == 2) return sweep_batched_dispatch<1, 2>(v, cases, work, nwork, parity, s);
-    if (form == 1) return sweep_batched_dispatch<1, 1>(v, cases, work, nwork, parity, s);
-    return sweep_batched_dispatch<1, 0>(v, cases, work, nwork, parity, s);
+    if (form == 2) return with_shape<1, 2>(v, f);
+    if (form == 1) return with_shape<1, 1>(v, f);
+    return with_shape<1, 0>(v, f);
   }
-  if (form == 2) return sweep_batched_dispatch<2, 2>(v, cases, work, nwork, parity, s);
-  if (form == 1) return sweep_batched_dispatch<2, 1>(v, cases, work, nwork, parity, s);
-  return sweep_batched_dispatch<2, 0>(v, cases, work, nwork, parity, s);
+  if (form == 2) return with_shape<2, 2>(v, f);
+  if (form == 1) return with_shape<2, 1>(v, f);
+  return with_shape<2, 0>(v, f);
 }
 
-cudaError_t launch_sweep_persistent(int nh, int form, const BatchCase *cases, const WorkItem *work, int nwork,
+cudaError_t sweep_batched_slots(int nh, int form, int v, bool persistent, int *ctas) {
+  return with_sweep(nh, form, v, [&](auto k) { return decltype(k)::slots(persistent, ctas); });
+}
+
+cudaError_t launch_sweep_batched(int nh, int form, const BatchCase *cases, const WorkItem *work, int nwork, int grid,
+                                 int parity, cudaStream_t s, int v) {
+  return with_sweep(nh, form, v, [&](auto k) { return decltype(k)::step(cases, work, nwork, grid, parity, s); });
+}
+
+cudaError_t launch_sweep_persistent(int nh, int form, const BatchCase *cases, const WorkItem *work, int nwork, int grid,
                                     int parity0, int nsteps, GridSync *sync, long long spin_limit, cudaStream_t s,
-                                    int v, int *grid) {
+                                    int v, int *launched) {
   if (v < 0 || v >= sweep_batched_count(nh)) return cudaErrorInvalidValue;
-  if (nh == 1) {
-    if (form == 2) return sweep_persistent_dispatch<1, 2>(v, cases, work, nwork, parity0, nsteps, sync, spin_limit, s, grid);
-    if (form == 1) return sweep_persistent_dispatch<1, 1>(v, cases, work, nwork, parity0, nsteps, sync, spin_limit, s, grid);
-    return sweep_persistent_dispatch<1, 0>(v, cases, work, nwork, parity0, nsteps, sync, spin_limit, s, grid);
-  }
-  if (form == 2) return sweep_persistent_dispatch<2, 2>(v, cases, work, nwork, parity0, nsteps, sync, spin_limit, s, grid);
-  if (form == 1) return sweep_persistent_dispatch<2, 1>(v, cases, work, nwork, parity0, nsteps, sync, spin_limit, s, grid);
-  return sweep_persistent_dispatch<2, 0>(v, cases, work, nwork, parity0, nsteps, sync, spin_limit, s, grid);
+  return with_sweep(nh, form, v, [&](auto k) {
+    return decltype(k)::persistent(cases, work, nwork, grid, parity0, nsteps, sync, spin_limit, s, launched);
+  });
 }
 
 cudaError_t launch_sweep_step(const DevParams &P, const FusedBuffers &B, cudaStream_t s, int v) {
