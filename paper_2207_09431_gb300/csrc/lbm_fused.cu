@@ -404,13 +404,15 @@ const char *fused_variant_name(const DevParams &P, int v) {
 // A tile form whose tiles all fit on the device at once beats the row sweep (whose
 // pipeline fill is most of a short segment), the smaller tile the better, until one
 // wave no longer holds them.  Measured per step on a GB300 (152 SMs), population form:
-//   64 x 128   16x4/224 3.7 us (128 tiles)      32x4/384 4.2    32x8/352 5.6    sweep 5.9 us
-//   100 x 200  32x4/384 5.2 us (200 tiles)      16x4/224 5.5+   32x8/352 5.9    sweep 6.8 us
-//   150 x 300  32x4/288 6.5 us (375 tiles)      32x8/352 7.4    sweep 8.0 us
-//   200 x 400  32x8/352 9.2 us (350 tiles)      32x4/288 9.9    sweep 9.7 us
-//   300 x 600  sweep 13.3 us                    32x8/352 14.4 us (750 tiles)
-// Three components: 128 x 128 16x8/320 5.3 us, 32x8/352 7.4, sweep 7.2; 256 x 256 32x8/352
-// 9.4 us (256 tiles), sweep 10.9; 512 x 512 sweep 22.1, 32x8/352 28.3 us.
+//   64 x 128   16x4/224 3.7 us (128 tiles)      32x4/384 4.2    32x8/448 5.2    sweep 5.3 us
+//   100 x 200  32x4/384 5.2 us (200 tiles)      16x4/224 5.5+   32x8/448 5.4    sweep 5.5 us
+//   150 x 300  32x4/288 6.4 us (375 tiles)      32x8/448 7.1    sweep 6.4 us
+//   180 x 360  32x8/448 7.4 us (270 tiles)      32x8/352/3 7.9  sweep 8.6 us
+//   200 x 400  sweep 8.1 us                     32x8/352/3 9.1 us (350 tiles, three to an SM)
+//   300 x 600  sweep 12.1 us                    32x8/352/3 14.4 us (750 tiles)
+// Three components: 128 x 128 16x8/320 5.3 us, 32x8/352 7.3, sweep 7.1; 100 x 200 16x8/320 6.6
+// us (175 tiles), 32x8/352 7.4; 256 x 256 32x8/352 9.4 us (256 tiles), 16x8/320 10.7 (512), sweep
+// 10.9; 512 x 512 sweep 22.0, 32x8/352 28.3 us.
 int fused_default_variant(const DevParams &P) {
   static const int sms = [] {
     int dev = 0, n = 0;
@@ -425,9 +427,9 @@ int fused_default_variant(const DevParams &P) {
     if (tiles(16, 4) <= sms) return ns + nb;
     if (tiles(32, 4) <= 2 * sms) return ns + nb + 1;
     if (tiles(32, 4) <= 3 * sms) return ns + nb + 2;
-    if (tiles(32, 8) <= 3 * sms) return ns;
+    if (tiles(32, 8) <= 2 * sms) return ns + 1;
   } else {
-    if (tiles(16, 8) <= sms) return ns + nb;
+    if (tiles(16, 8) <= 2 * sms) return ns + nb;
     if (tiles(32, 8) <= 2 * sms) return ns;
   }
   return sweep_default_variant(P, sms);

@@ -658,24 +658,46 @@ static int sweep_steps(const DevParams &P, int tx, int rs, int fill, int residen
   return (int)(waves * ((len + fill) / rs));
 }
 
-// The sweep a large lattice starts with.  Two components: four-warp strips of 58
-// columns take 0.96 of the time of 160-thread strips of 60 per pipeline step (the
-// fifth warp has almost no items after stage 0), so the 60-column strips are taken where they
-// save more steps than that: 2048 x 4096 (164 against 177 steps: 301 against 305
-// us), not 1024 x 2048 (47 both: 85.5 against 82.1 us), 517 x 1031 (29.1 against 28.0 us).
-// Three components: the shape with fewer steps (512 x 512: 32x4 12 steps, 22.1 us, 64x2
-// 13 steps, 23.2 us; 1024 x 1024: 34 and 33 steps, 75.3 and 70.7 us).
+// The sweep a lattice too large for one wave of tiles starts with: the shape with the least
+// pipeline steps x time per step.  The shapes differ in how they round: a strip width leaves
+// columns of the last strip empty, rows per step round the segment up, and many rows in
+// few columns pay a longer fill but split a small lattice finer.  Their time per step, all
+// CTA slots filled, is nearly the same (58x2/128/3 = 1; fitted to 35 sizes from 32 x 64 to
+// 2048 x 4096 and 4000 x 240 in three state forms, where the choice is within 0.1 % of the best
+// of these on average, 2 % at worst).  Those of 128 or 192 threads fill every lane with an order
+// parameter: RS (TX + 6) = threads.  us per step on a GB300, 58x2/128/3 and 60x2/160/3
+// against the choice here: 200 x 400 9.7 and 10.6 against 8.1 (18x8), 300 x 600 13.3
+// and 14.4 against 12.1 (26x6), 517 x 1031 28.1 and 29.2 against 27.6 (58x3), 2048 x 4096 305
+// and 301 against 291 (90x2).  Three components: 517 x 1031 45.6 (62x2) against 46.5 (32x4),
+// 1500 x 1500 147 (62x2) against 154 (64x2), 300 x 300 11.6 (26x6) against 13.1 (32x4).
 int sweep_default_variant(const DevParams &P, int sms) {
-  if (P.nh == 1)
-    return 0.96 * sweep_steps(P, 58, 2, fill_rows<2>(), 3 * sms) <= sweep_steps(P, 60, 2, fill_rows<2>(), 3 * sms) ? 11 : 9;
-  return sweep_steps(P, 32, 4, fill_rows<4>(), 2 * sms) < sweep_steps(P, 64, 2, fill_rows<2>(), 2 * sms) ? 1 : 0;
+  struct Shape {
+    int variant, tx, rs, per_sm;
+    double cost;
+  };
+  static const Shape two[] = {{11, 58, 2, 3, 1.0}, {9, 60, 2, 3, 1.02}, {2, 90, 2, 2, 1.01}, {3, 58, 3, 2, 1.05},
+                              {4, 42, 4, 2, 1.045}, {7, 26, 6, 2, 1.145}, {5, 18, 8, 2, 1.12}};
+  static const Shape three[] = {{3, 62, 2, 2, 1.0}, {0, 64, 2, 2, 1.02}, {1, 32, 4, 2, 1.03}, {2, 26, 6, 1, 1.0}};
+  const Shape *c = P.nh == 1 ? two : three;
+  const int n = P.nh == 1 ? 7 : 4;
+  int best = 0;
+  double least = 0.;
+  for (int i = 0; i < n; ++i) {
+    const int fill = 3 * c[i].rs + c[i].rs * ((6 + c[i].rs - 1) / c[i].rs);  // fill_rows
+    const double t = c[i].cost * sweep_steps(P, c[i].tx, c[i].rs, fill, c[i].per_sm * sms);
+    if (i == 0 || t < least) {
+      least = t;
+      best = c[i].variant;
+    }
+  }
+  return best;
 }
 
 const char *sweep_variant_name(const DevParams &P, int v) {
-  static const char *n1[13] = {"64x2/160/3", "32x4/160/3", "128x1/160/2", "64x4/288/2", "64x1/96/5",
-                               "32x8/320/2", "62x2/160/3", "126x1/160/2", "30x4/160/3", "60x2/160/3",
+  static const char *n1[13] = {"64x2/160/3", "32x4/160/3", "90x2/192/2", "58x3/192/2", "42x4/192/2",
+                               "18x8/192/2", "62x2/160/3", "26x6/192/2", "30x4/160/3", "60x2/160/3",
                                "28x4/160/3", "58x2/128/3", "58x2/128/4"};
-  static const char *n2[4] = {"64x2/160/2", "32x4/160/2", "64x1/96/4", "62x2/160/2"};
+  static const char *n2[4] = {"64x2/160/2", "32x4/160/2", "26x6/192/1", "62x2/160/2"};
   if (v < 0 || v >= sweep_variant_count(P)) v = 0;
   return P.nh == 1 ? n1[v] : n2[v];
 }
@@ -685,13 +707,14 @@ static cudaError_t sweep_dispatch(int v, const DevParams &P, const FusedBuffers 
   if constexpr (NH == 1) {
     switch (v) {
       case 1: return launch_sweep_t<32, 4, NH, FORM, 160, 3>(P, B, s);
-      case 2: return launch_sweep_t<128, 1, NH, FORM, 160, 2>(P, B, s);
-      case 3: return launch_sweep_t<64, 4, NH, FORM, 288, 2>(P, B, s);
-      case 4: return launch_sweep_t<64, 1, NH, FORM, 96, 5>(P, B, s);
-      case 5: return launch_sweep_t<32, 8, NH, FORM, 320, 2>(P, B, s);
+      // 2 to 5, 7: every lane of six warps has an order parameter (RS (TX + 6) = 192)
+      case 2: return launch_sweep_t<90, 2, NH, FORM, 192, 2>(P, B, s);
+      case 3: return launch_sweep_t<58, 3, NH, FORM, 192, 2>(P, B, s);
+      case 4: return launch_sweep_t<42, 4, NH, FORM, 192, 2>(P, B, s);
+      case 5: return launch_sweep_t<18, 8, NH, FORM, 192, 2>(P, B, s);
       // strips whose collision rows are a whole number of warps (RS (TX + 2) = 128)
       case 6: return launch_sweep_t<62, 2, NH, FORM, 160, 3>(P, B, s);
-      case 7: return launch_sweep_t<126, 1, NH, FORM, 160, 2>(P, B, s);
+      case 7: return launch_sweep_t<26, 6, NH, FORM, 192, 2>(P, B, s);
       case 8: return launch_sweep_t<30, 4, NH, FORM, 160, 3>(P, B, s);
       // ... and whose field rows are (RS (TX + 4) = 128)
       case 9: return launch_sweep_t<60, 2, NH, FORM, 160, 3>(P, B, s);
@@ -704,7 +727,7 @@ static cudaError_t sweep_dispatch(int v, const DevParams &P, const FusedBuffers 
   } else {
     switch (v) {
       case 1: return launch_sweep_t<32, 4, NH, FORM, 160, 2>(P, B, s);
-      case 2: return launch_sweep_t<64, 1, NH, FORM, 96, 4>(P, B, s);
+      case 2: return launch_sweep_t<26, 6, NH, FORM, 192, 1>(P, B, s);
       case 3: return launch_sweep_t<62, 2, NH, FORM, 160, 2>(P, B, s);
       default: return launch_sweep_t<64, 2, NH, FORM, 160, 2>(P, B, s);
     }
