@@ -222,6 +222,7 @@ def kernel_bytes_per_node(nh: int) -> dict:
     return {
         "k_fields_step": f * (9 * nh + 9 + 1 + nh + 3 + 3 + 1 + 1),
         "k_collide_step": f * (9 + nh + 3 + 1 + 2 + 1 + nh + 9 + 9 * nh),
+        "k_collide_push": f * (9 + nh + 3 + 1 + 2 + 1 + nh + 9 + 9 * nh),
     }
 
 

@@ -498,9 +498,10 @@ lbm_status lbm_load(lbm_handle *h, const char *path) {
 int lbm_kernels_per_step(const lbm_handle *h) { return h ? h->kernels_per_step() : 0; }
 
 const char *lbm_kernel_name(const lbm_handle *h, int i) {
-  static const char *names[lbm::kSplitKernels] = {"k_fields_step", "k_collide_step"};
+  static const char *open_ends[lbm::kSplitKernels] = {"k_fields_step", "k_collide_step"};
+  static const char *periodic_x[lbm::kSplitKernels] = {"k_fields_step", "k_collide_push"};
   if (!h || i < 0 || i >= h->kernels_per_step()) return "";
-  if (!h->fused()) return names[i];
+  if (!h->fused()) return h->dp.open_x ? open_ends[i] : periodic_x[i];
   lbm_handle *m = const_cast<lbm_handle *>(h);
   const bool sweep = h->variant < lbm::sweep_variant_count(h->dp);
   m->kname = std::string(sweep ? "k_step_sweep[" : "k_step_fused[") + lbm::fused_variant_name(h->dp, h->variant) + "]";

@@ -2,9 +2,9 @@
 // the mixed difference scheme and the open x boundaries:
 //   k_fields_step   C_i = sum_a h_a^i (Eq. 22), rho, mu (Eq. 5), u (Eq. 23),
 //                   p (Eq. 24/R3), new tau (Eq. 25-33)
-//   k_collide_step  S_i + V_i (Eq. 6, 18, 21), collision of g (Eq. 14) and h (Eq.
-//                   18), streaming with half-way bounce-back or the open boundaries,
-//                   the destination-side source term (R9)
+//   k_collide_push  S_i + V_i (Eq. 6, 18, 21), collision of g (Eq. 14) and h (Eq.
+//   k_collide_step  18), streaming with half-way bounce-back and (the latter) the open
+//                   boundaries, the destination-side source term (R9)
 // The fields between the two live in scratch planes carved from the caller's
 // arena.  All arithmetic FP32.  Also the macro fields, the initial equilibria and
 // the observables.
@@ -249,14 +249,11 @@ __device__ __forceinline__ long long tile_node(const DevParams &P, int x, int y)
 // ring slot, where a node's stencils of up to 25 points used to read the planes through
 // L1 and form rho again at every point.  The kernels were four (moments, fields, sources,
 // collision) and, with open ends, a fifth that walked the boundary rows: the
-// sources and the open ends are now part of the collision kernel, whose post-collision
-// populations of the tile and its one-node ring stay in shared memory and are
-// gathered by the node they arrive at (coalesced stores; the ring's collisions, a third
-// more, are computed twice).  Bound by the latency of two short kernels on small
-// lattices and by instruction issue on large ones.  Measured on a GB300, one step in
-// a replayed graph, two kernels against four (five): mixed scheme 64 x 128 11.0 against
-// 22.3 us, 200 x 400 18.0 against 29.6 us, 1024 x 2048 223 against 431 us; open channel
-// 240 x 60 11.0 against 31.2 us.  Tiles of 8 rows (fewer collisions twice, fewer CTAs)
+// sources and the open ends are now part of the collision kernel.  Bound by the latency of two
+// short kernels on small lattices and by instruction issue on large ones.  Measured on a
+// GB300, one step in a replayed graph, two kernels against four (five): mixed scheme 64 x 128
+// 10.7 against 22.3 us, 200 x 400 14.2 against 29.6 us, 1024 x 2048 182 against 431 us; open
+// channel 240 x 60 11.0 against 31.2 us.  Tiles of 8 rows (fewer collisions twice, fewer CTAs)
 // ran 1 to 5 % slower above 400 x 800 at their best register budget and up to 10 % slower
 // on small lattices.  The order of a node's operations is that of the earlier kernels.
 constexpr int kTileX = 32, kTileY = 4;
@@ -383,6 +380,52 @@ __device__ __forceinline__ float source_of(const DevParams &P, int i, const floa
   return D0s * lapmu;
 }
 
+// Post-collision populations of a node whose u, mu and stencil values (at) are in place:
+// sv its sources, gv its g, tn its new relaxation time; put(a, g*_a, h*) takes them.
+// With tau_h = 1/2 the BGK step of Eq. 18 replaces h by its modified equilibrium:
+// h* = C Gamma + Phi/2 + SV Gamma/2.
+template <int NH, int SCHEME, typename Reader, typename Put>
+__device__ __forceinline__ void collide_node(const DevParams &P, NodeCtx &n, const Reader &at, const float (&sv)[NH],
+                                             const float (&gv)[9], float tn, const Put &put) {
+  gather_gradients(SCHEME, at, n);
+  n.Fs[0] = n.mu[0] * n.gC[0][0] + n.mu[1] * n.gC[1][0] + n.mu[2] * n.gC[2][0];
+  n.Fs[1] = n.mu[0] * n.gC[0][1] + n.mu[1] * n.gC[1][1] + n.mu[2] * n.gC[2][1];
+  n.Fb[0] = P.force_x;
+  n.Fb[1] = -n.rho * P.gravity;
+  const float omega = 1.0f / (tn + 0.5f);
+#pragma unroll
+  for (int a = 0; a < 9; ++a) {
+    const float G = gamma_a(a, n.ux, n.uy);
+    // (which product of the equilibrium is rounded on its own is spelled out: left to the
+    // compiler it changes with the code around it, and the results by rounding)
+    const float pg = phi_g(n, a, G), Gw = G - wt(a), rc = n.rho * kCs2;
+    const float lin = a < 5 ? __fmaf_rn(wt(a), n.p, __fmul_rn(rc, Gw)) : __fmaf_rn(rc, Gw, __fmul_rn(wt(a), n.p));
+    const float geq = lin - 0.5f * pg;
+    float hs[NH];
+#pragma unroll
+    for (int i = 0; i < NH; ++i) {
+      const float ph = phi_h(n, i, a, G);
+      hs[i] = n.C[i] * G + 0.5f * ph + 0.5f * sv[i] * G;
+    }
+    put(a, gv[a] - omega * (gv[a] - geq) + pg, hs);
+  }
+}
+
+// C, rho and p around node (lx, ly) of a tile.
+template <int NH, typename S, typename RC>
+struct StencilReader {
+  const S &s;
+  int lx, ly;
+  __device__ __forceinline__ int q(int dx, int dy) const { return RC::slot(lx + dx, ly + dy); }
+  __device__ __forceinline__ void C(int dx, int dy, float c[3]) const {
+    c[0] = s.C[0][q(dx, dy)];
+    c[1] = NH == 2 ? s.C[NH - 1][q(dx, dy)] : 0.0f;
+    c[2] = 1.0f - c[0] - c[1];
+  }
+  __device__ __forceinline__ float rho(int dx, int dy, const float *) const { return s.rho[q(dx, dy)]; }
+  __device__ __forceinline__ float p(int dx, int dy) const { return s.p[q(dx, dy)]; }
+};
+
 template <int NH, int SCHEME>
 struct CollideSmem {
   using RC = Ring<2 + SCHEME>;
@@ -394,10 +437,10 @@ struct CollideSmem {
 // Threads: the collisions of the tile and its ring in one pass.
 constexpr int kCollideThreads = (Ring<1>::N + 31) / 32 * 32;
 
-// Sources, collision and streaming of a tile.  With tau_h = 1/2 the BGK step of
-// Eq. 18 replaces h by its modified equilibrium, so h itself is read at the outlet only:
-// h* = C Gamma + Phi/2 + SV Gamma/2.  Populations that would cross a wall return in
-// the opposite direction.  Open x: at the inlet (x = 0, e_x = +1) g comes from a ghost
+// Sources, collision and streaming of a tile with open x boundaries: the populations of
+// the tile and its ring meet in shared memory and are gathered by the node they arrive at
+// (an outlet node needs all of its own at once).  Populations that would cross a wall return in
+// the opposite direction.  At the inlet (x = 0, e_x = +1) g comes from a ghost
 // column x = -1 whose post-collision g is the equilibrium w p + rho cs^2 (Gamma - w) at
 // (u_in, 0) plus the non-equilibrium part of column 0's post-collision g, h the
 // equilibrium c_in Gamma(u_in) plus the node's destination-side term; at the outlet
@@ -421,7 +464,7 @@ __global__ void __launch_bounds__(kCollideThreads, MINB)
 
   // this thread's node of the one-node ring (real rows, and columns of the lattice)
   const int lx = t % R1::W - 1, ly = t / R1::W - 1, xr = x0 + lx, yr = y0 + ly;
-  const bool ring = t < R1::N && (P.periodic_y || (yr >= 0 && yr < P.ny)) && (!P.open_x || (xr >= 0 && xr < P.nx));
+  const bool ring = t < R1::N && (P.periodic_y || (yr >= 0 && yr < P.ny)) && xr >= 0 && xr < P.nx;
   const bool inside = tile_inside(P, x0, y0, 2 + SCHEME);
   const long long kr = inside ? node_index(P, xr, yr) : tile_node(P, xr, yr);
   NodeCtx n;
@@ -451,18 +494,7 @@ __global__ void __launch_bounds__(kCollideThreads, MINB)
   __syncthreads();
 
   if (ring) {
-    struct {
-      const S &s;
-      int lx, ly;
-      __device__ __forceinline__ int q(int dx, int dy) const { return RC::slot(lx + dx, ly + dy); }
-      __device__ __forceinline__ void C(int dx, int dy, float c[3]) const {
-        c[0] = s.C[0][q(dx, dy)];
-        c[1] = NH == 2 ? s.C[NH - 1][q(dx, dy)] : 0.0f;
-        c[2] = 1.0f - c[0] - c[1];
-      }
-      __device__ __forceinline__ float rho(int dx, int dy, const float *) const { return s.rho[q(dx, dy)]; }
-      __device__ __forceinline__ float p(int dx, int dy) const { return s.p[q(dx, dy)]; }
-    } at{s, lx, ly};
+    const StencilReader<NH, S, RC> at{s, lx, ly};
     float sv[NH];
 #pragma unroll
     for (int i = 0; i < NH; ++i) {
@@ -477,27 +509,11 @@ __global__ void __launch_bounds__(kCollideThreads, MINB)
     }
     s.ux[t] = n.ux;
     s.uy[t] = n.uy;
-    gather_gradients(SCHEME, at, n);
-    n.Fs[0] = n.mu[0] * n.gC[0][0] + n.mu[1] * n.gC[1][0] + n.mu[2] * n.gC[2][0];
-    n.Fs[1] = n.mu[0] * n.gC[0][1] + n.mu[1] * n.gC[1][1] + n.mu[2] * n.gC[2][1];
-    n.Fb[0] = P.force_x;
-    n.Fb[1] = -n.rho * P.gravity;
-    const float omega = 1.0f / (tn + 0.5f);
+    collide_node<NH, SCHEME>(P, n, at, sv, gv, tn, [&](int a, float gs, const float (&hs)[NH]) {
+      s.g[a][t] = gs;
 #pragma unroll
-    for (int a = 0; a < 9; ++a) {
-      const float G = gamma_a(a, n.ux, n.uy);
-      // (which product of the equilibrium is rounded on its own is spelled out: left to the
-      // compiler it changes with the code around it, and the results by rounding)
-      const float pg = phi_g(n, a, G), Gw = G - wt(a), rc = n.rho * kCs2;
-      const float lin = a < 5 ? __fmaf_rn(wt(a), n.p, __fmul_rn(rc, Gw)) : __fmaf_rn(rc, Gw, __fmul_rn(wt(a), n.p));
-      const float geq = lin - 0.5f * pg;
-      s.g[a][t] = gv[a] - omega * (gv[a] - geq) + pg;
-#pragma unroll
-      for (int i = 0; i < NH; ++i) {
-        const float ph = phi_h(n, i, a, G);
-        s.h[i][a][t] = n.C[i] * G + 0.5f * ph + 0.5f * sv[i] * G;
-      }
-    }
+      for (int i = 0; i < NH; ++i) s.h[i][a][t] = hs[i];
+    });
   }
   __syncthreads();
 
@@ -510,7 +526,7 @@ __global__ void __launch_bounds__(kCollideThreads, MINB)
   float gy[9];
   unsigned entered = 0;  // outlet: directions that enter there
   float wsum = 0.f, U = 0.f, inv = 1.f;
-  const bool outlet = P.open_x && x == P.nx - 1;
+  const bool outlet = x == P.nx - 1;
   if (outlet) {
     U = fminf(fmaxf(ux, 0.0f), 1.0f);
     inv = 1.0f / (1.0f + U);
@@ -526,7 +542,7 @@ __global__ void __launch_bounds__(kCollideThreads, MINB)
 #pragma unroll
       for (int i = 0; i < NH; ++i)
         h_out[pop_index(k, i * 9 + a, 9 * NH)] = s.h[i][opp(a)][q0] + 0.5f * s.sv[i][q0] * G;
-    } else if (P.open_x && sx < 0) {
+    } else if (sx < 0) {
       const int q = R1::slot(tx, ty - ey(a));  // column 0 of the source row
       const int qc = RC::slot(tx, ty - ey(a));
       const float rho = s.rho[qc], p = s.p[qc], w = wt(a);
@@ -539,7 +555,7 @@ __global__ void __launch_bounds__(kCollideThreads, MINB)
 #pragma unroll
       for (int i = 0; i < NH; ++i)
         h_out[pop_index(k, i * 9 + a, 9 * NH)] = P.c_in[i] * Gin + 0.5f * s.sv[i][q0] * G;
-    } else if (P.open_x && sx >= P.nx) {
+    } else if (sx >= P.nx) {
       const int q = R1::slot(tx, ty - ey(a));       // column nx - 1 of the source row
       const int qi = R1::slot(tx - 1, ty);          // (nx - 2, y), where its population arrives
       entered |= 1u << a;
@@ -570,6 +586,102 @@ __global__ void __launch_bounds__(kCollideThreads, MINB)
   }
 #pragma unroll
   for (int a = 0; a < 9; ++a) g_out[pop_index(k, a, 9)] = gy[a];
+}
+
+// Sources, collision and streaming of a tile where x is periodic: every node collides
+// once and stores its populations at the nodes they arrive at, whose sources and
+// velocity (for the term of R9) are in the tile's ring.  The gather form above
+// collides the ring as well, 204 nodes for 128; here the ring costs its sources only, and the
+// stencils of a node reach two nodes instead of three.  One row's stores stay
+// together, shifted by a column in the six directions with e_x.  Bound by instruction issue.
+// Against the gather form (which this scheme took as well), us per step: 200 x 400 18.0 -> 14.2,
+// 1024 x 2048 225 -> 182 (157 -> 113 in this kernel), three components 256 x 256 18.3 -> 14.5.
+// Five or six CTAs per SM (fewer registers) are within 2 % of the four asked for.
+template <int NH>
+struct PushSmem {
+  using R2 = Ring<2>;
+  using R1 = Ring<1>;
+  float C[NH][R2::N], rho[R2::N], p[R2::N], mu[NH][R2::N];
+  float sv[NH][R1::N], ux[R1::N], uy[R1::N];
+};
+template <int NH, int SCHEME, int MINB>
+__global__ void __launch_bounds__(kTileX *kTileY, MINB)
+    k_collide_push(DevParams P, const float *__restrict__ g, const float *__restrict__ Cf,
+                   const float *__restrict__ mu, const float *__restrict__ pf, const float *__restrict__ uxf,
+                   const float *__restrict__ uyf, const float *__restrict__ tau_new, float *__restrict__ SV,
+                   float *__restrict__ g_out, float *__restrict__ h_out) {
+  using S = PushSmem<NH>;
+  using R2 = typename S::R2;
+  using R1 = typename S::R1;
+  constexpr int NT = kTileX * kTileY;
+  __shared__ S s;
+  const int t = threadIdx.x, x0 = blockIdx.x * kTileX, y0 = blockIdx.y * kTileY;
+  const int tx = t % kTileX, ty = t / kTileX, x = x0 + tx, y = y0 + ty;
+  const bool mine = x < P.nx && y < P.ny;
+  const long long k = node_index(P, x, y);
+  NodeCtx n;
+  float gv[9], tn = 0.f;
+  if (mine) {
+#pragma unroll
+    for (int a = 0; a < 9; ++a) gv[a] = g[pop_index(k, a, 9)];
+    tn = tau_new[k];
+#pragma unroll
+    for (int j = 0; j < 3; ++j) n.mu[j] = mu[(long long)j * P.plane + k];
+  }
+  const bool inside = tile_inside(P, x0, y0, 2);
+  for (int q = t; q < R2::N; q += NT) {
+    const int cx = q % R2::W - 2, cy = q / R2::W - 2;
+    const long long kq = inside ? node_index(P, x0 + cx, y0 + cy) : tile_node(P, x0 + cx, y0 + cy);
+    const float c0 = Cf[kq], c1 = NH == 2 ? Cf[P.plane + kq] : 0.0f;
+    s.C[0][q] = c0;
+    if (NH == 2) s.C[NH - 1][q] = c1;
+    s.rho[q] = rho_of(P, c0, c1, 1.0f - c0 - c1);
+    s.p[q] = pf[kq];
+#pragma unroll
+    for (int i = 0; i < NH; ++i) s.mu[i][q] = mu[(long long)i * P.plane + kq];
+    if (cx >= -1 && cx <= kTileX && cy >= -1 && cy <= kTileY) {
+      s.ux[R1::slot(cx, cy)] = uxf[kq];
+      s.uy[R1::slot(cx, cy)] = uyf[kq];
+    }
+  }
+  __syncthreads();
+  for (int q = t; q < R1::N; q += NT) {
+    const int lx = q % R1::W - 1, ly = q / R1::W - 1;
+    if (!P.periodic_y && (y0 + ly < 0 || y0 + ly >= P.ny)) continue;  // beyond a wall nothing arrives
+#pragma unroll
+    for (int i = 0; i < NH; ++i) {
+      float cv[9], mv[9];
+#pragma unroll
+      for (int a = 0; a < 9; ++a) {
+        cv[a] = s.C[i][R2::slot(lx + ex(a), ly + ey(a))];
+        mv[a] = s.mu[i][R2::slot(lx + ex(a), ly + ey(a))];
+      }
+      s.sv[i][q] = source_of(P, i, cv, mv);
+    }
+  }
+  __syncthreads();
+  if (!mine) return;
+  const int q0 = R1::slot(tx, ty);
+  float sv[NH];
+#pragma unroll
+  for (int i = 0; i < NH; ++i) {
+    sv[i] = s.sv[i][q0];
+    SV[(long long)i * P.plane + k] = sv[i];
+  }
+  n.ux = s.ux[q0];
+  n.uy = s.uy[q0];
+  const StencilReader<NH, S, R2> at{s, tx, ty};
+  const bool last_row = !P.periodic_y && y == P.ny - 1, first_row = !P.periodic_y && y == 0;
+  collide_node<NH, SCHEME>(P, n, at, sv, gv, tn, [&](int a, float gs, const float (&hs)[NH]) {
+    // half-way bounce-back: back to this node, in the opposite direction
+    const bool back = (ey(a) > 0 && last_row) || (ey(a) < 0 && first_row);
+    const int b = back ? opp(a) : a, q = back ? q0 : R1::slot(tx + ex(a), ty + ey(a));
+    const long long kd = back ? k : node_index(P, wrap_x(x + ex(a), P.nx), wrap_y(y + ey(a), P.ny, 1));
+    const float G = back ? gamma_a(opp(a), s.ux[q], s.uy[q]) : gamma_a(a, s.ux[q], s.uy[q]);
+    g_out[pop_index(kd, b, 9)] = gs;
+#pragma unroll
+    for (int i = 0; i < NH; ++i) h_out[pop_index(kd, i * 9 + b, 9 * NH)] = hs[i] + 0.5f * s.sv[i][q] * G;
+  });
 }
 
 // Modified equilibria (Eq. 16, 20) of given C, p, u, and tau at zero strain rate
@@ -912,7 +1024,7 @@ static dim3 node_grid(const DevParams &P, dim3 blk) {
   return dim3((P.nx + blk.x - 1) / blk.x, (P.ny + blk.y - 1) / blk.y);
 }
 
-template <int NH, int SCHEME, int MINB>
+template <int NH, int SCHEME>
 static cudaError_t split_step(const DevParams &P, const StepBuffers &B, cudaStream_t s, cudaEvent_t *ev) {
   using S = CollideSmem<NH, SCHEME>;
   static_assert(sizeof(S) <= 48 * 1024, "no opt-in for more shared memory");
@@ -921,15 +1033,21 @@ static cudaError_t split_step(const DevParams &P, const StepBuffers &B, cudaStre
   k_fields_step<NH, SCHEME><<<grd, kTileX * kTileY, 0, s>>>(P, B.h_in, B.g_in, B.tau_in, B.C, B.mu, B.p, B.ux, B.uy,
                                                            B.tau_out, B.shear, B.err);
   if (ev) cudaEventRecord(ev[1], s);
-  k_collide_step<NH, SCHEME, MINB><<<grd, kCollideThreads, sizeof(S), s>>>(
-      P, B.g_in, B.h_in, B.C, B.mu, B.p, B.ux, B.uy, B.tau_out, B.SV, B.g_out, B.h_out);
+  if (P.open_x)
+    k_collide_step<NH, SCHEME, NH == 1 ? 4 : 2><<<grd, kCollideThreads, sizeof(S), s>>>(
+        P, B.g_in, B.h_in, B.C, B.mu, B.p, B.ux, B.uy, B.tau_out, B.SV, B.g_out, B.h_out);
+  else if constexpr (SCHEME == 1)  // (periodic x with central differences takes the one-kernel forms)
+    k_collide_push<NH, SCHEME, NH == 1 ? 4 : 2><<<grd, kTileX * kTileY, 0, s>>>(P, B.g_in, B.C, B.mu, B.p, B.ux, B.uy, B.tau_out,
+                                                                  B.SV, B.g_out, B.h_out);
+  else
+    return cudaErrorNotSupported;
   if (ev) cudaEventRecord(ev[2], s);
   return cudaGetLastError();
 }
 
 cudaError_t launch_split_step(const DevParams &P, const StepBuffers &B, cudaStream_t s, cudaEvent_t *ev) {
-  if (P.nh == 1) return P.fd_scheme == 1 ? split_step<1, 1, 4>(P, B, s, ev) : split_step<1, 0, 4>(P, B, s, ev);
-  return P.fd_scheme == 1 ? split_step<2, 1, 2>(P, B, s, ev) : split_step<2, 0, 2>(P, B, s, ev);
+  if (P.nh == 1) return P.fd_scheme == 1 ? split_step<1, 1>(P, B, s, ev) : split_step<1, 0>(P, B, s, ev);
+  return P.fd_scheme == 1 ? split_step<2, 1>(P, B, s, ev) : split_step<2, 0>(P, B, s, ev);
 }
 
 void launch_macros(const DevParams &P, const StepBuffers &B, cudaStream_t s) {
