@@ -207,10 +207,10 @@ struct lbm_handle {
   long long prev_step;
   double prev_v, y_int;
   std::string last_error;
-  // captured runs of kStepGraph steps without diagnostics, one per starting
-  // buffer (cur), for the launch configuration they were captured with
-  cudaGraphExec_t graph[2] = {nullptr, nullptr};
-  int graph_variant[2] = {-1, -1};
+  // captured run of kStepGraph steps without diagnostics, for the starting buffer (cur)
+  // and the launch configuration it was captured with
+  cudaGraphExec_t graph = nullptr;
+  int graph_variant = -1, graph_from = -1;
   static constexpr int kStepGraph = 16;
   // lbm_set_fields: a stream of its own for the upload of C in row chunks,
   // overlapped with the conversion and initial equilibria on `stream`
@@ -219,8 +219,7 @@ struct lbm_handle {
   cudaEvent_t upload_ev[kUploadChunks + 1] = {};
 
   ~lbm_handle() {
-    for (auto &g : graph)
-      if (g) cudaGraphExecDestroy(g);
+    if (graph) cudaGraphExecDestroy(graph);
     for (auto &e : upload_ev)
       if (e) cudaEventDestroy(e);
     if (copy_stream) cudaStreamDestroy(copy_stream);
