@@ -236,45 +236,49 @@ lbm_status lbm_step(lbm_handle *h, long long nsteps) {
   cudaError_t e = cudaMemsetAsync(h->err, 0, sizeof(unsigned), h->stream);
   if (e != cudaSuccess) return h->cuda_fail(e, "lbm_step memset");
   long long t = 0;
-  // Runs of kStepGraph steps are replayed from a captured graph (on a created
-  // stream; capture needs one).  The last step writes the diagnostics and is
+  // Runs of 16 and (small lattices) of 4 steps are replayed from captured graphs (on a
+  // created stream; capture needs one).  The last step writes the diagnostics and is
   // launched directly; a first run with a new configuration is too, so that
-  // its kernels are configured outside the capture.  The graph starts from one of the two
+  // its kernels are configured outside the capture.  A graph starts from one of the two
   // buffers, and a call that comes with the state in the other one takes a direct step
   // first: with a graph per buffer, captured where the first direct step had led, a
   // program of equal even runs captured anew on every call (64 steps of 64 x 128:
-  // 333 -> 279 us, GB300).
+  // 333 -> 279 us, GB300).  A launch from the host takes some 6 us, longer than a step of a
+  // lattice of up to about 150 x 300 nodes (3.6 to 6.4 us), whose last 15 steps therefore go
+  // in fours (279 -> 254 us); with larger ones the host is ahead of the device anyway.
   const bool capturable = h->stream != nullptr && h->stream != cudaStreamLegacy && h->stream != cudaStreamPerThread;
-  const int K = lbm_handle::kStepGraph;
-  if (capturable && nsteps - 1 >= K) {
-    const bool captured = h->graph && h->graph_variant == h->variant;
-    if (!captured || h->graph_from != h->cur) {
+  const bool small = (long long)h->prm.nx * h->prm.ny <= lbm_handle::kSmallNodes;
+  for (auto &sg : h->graphs) {
+    if (!capturable || nsteps - 1 < sg.steps || (sg.steps < lbm_handle::kStepGraph && !small)) continue;
+    if (nsteps - 1 - t < sg.steps) continue;
+    const bool captured = sg.exec && sg.variant == h->variant;
+    if (captured ? sg.from != h->cur : t == 0) {
       h->launch_step(false, nullptr);
-      t = 1;
+      ++t;
     }
     if (!captured) {
       const int c = h->cur;
-      if (h->graph) cudaGraphExecDestroy(h->graph);
-      h->graph = nullptr;
+      if (sg.exec) cudaGraphExecDestroy(sg.exec);
+      sg.exec = nullptr;
       cudaGraph_t g = nullptr;
       e = cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeThreadLocal);
-      for (int k = 0; k < K && e == cudaSuccess; ++k) {
+      for (int k = 0; k < sg.steps && e == cudaSuccess; ++k) {
         h->launch_step(false, nullptr);
         e = cudaGetLastError();
       }
       cudaError_t ec = cudaStreamEndCapture(h->stream, &g);
       if (e == cudaSuccess) e = ec;
-      if (e == cudaSuccess) e = cudaGraphInstantiate(&h->graph, g, 0);
+      if (e == cudaSuccess) e = cudaGraphInstantiate(&sg.exec, g, 0);
       if (g) cudaGraphDestroy(g);
       h->cur = c;  // an even number of captured steps returns to the same buffer
       if (e != cudaSuccess) {
-        h->graph = nullptr;
+        sg.exec = nullptr;
         return h->cuda_fail(e, "lbm_step graph capture");
       }
-      h->graph_variant = h->variant;
-      h->graph_from = c;
+      sg.variant = h->variant;
+      sg.from = c;
     }
-    for (; nsteps - 1 - t >= K && e == cudaSuccess; t += K) e = cudaGraphLaunch(h->graph, h->stream);
+    for (; nsteps - 1 - t >= sg.steps && e == cudaSuccess; t += sg.steps) e = cudaGraphLaunch(sg.exec, h->stream);
     if (e != cudaSuccess) return h->cuda_fail(e, "lbm_step graph launch");
   }
   for (; t < nsteps; ++t) h->launch_step(t == nsteps - 1, nullptr);

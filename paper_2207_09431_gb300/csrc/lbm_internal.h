@@ -207,11 +207,15 @@ struct lbm_handle {
   long long prev_step;
   double prev_v, y_int;
   std::string last_error;
-  // captured run of kStepGraph steps without diagnostics, for the starting buffer (cur)
+  // captured runs of steps without diagnostics, each for the starting buffer (cur)
   // and the launch configuration it was captured with
-  cudaGraphExec_t graph = nullptr;
-  int graph_variant = -1, graph_from = -1;
+  struct StepGraph {
+    int steps, variant = -1, from = -1;
+    cudaGraphExec_t exec = nullptr;
+  };
   static constexpr int kStepGraph = 16;
+  static constexpr long long kSmallNodes = 45000;  // lattices whose steps are shorter than a launch
+  StepGraph graphs[2] = {{kStepGraph}, {4}};
   // lbm_set_fields: a stream of its own for the upload of C in row chunks,
   // overlapped with the conversion and initial equilibria on `stream`
   static constexpr int kUploadChunks = 4;
@@ -219,7 +223,8 @@ struct lbm_handle {
   cudaEvent_t upload_ev[kUploadChunks + 1] = {};
 
   ~lbm_handle() {
-    if (graph) cudaGraphExecDestroy(graph);
+    for (auto &sg : graphs)
+      if (sg.exec) cudaGraphExecDestroy(sg.exec);
     for (auto &e : upload_ev)
       if (e) cudaEventDestroy(e);
     if (copy_stream) cudaStreamDestroy(copy_stream);
