@@ -315,15 +315,15 @@ static cudaError_t launch_batched_t(const BatchCase *cases, const WorkItem *work
 template <int NH, int FORM>
 struct VariantTable {
   static constexpr int kBatched = FORM == 2 ? 2 : (NH == 1 ? 5 : 2);  // those that batches have too
-  // small tiles for small lattices (not in batches), after the others
-  static constexpr int kSmall = NH == 1 ? 3 : 2;
+  // tiles for small lattices (not in batches), after the others
+  static constexpr int kSmall = NH == 1 ? 3 : 4;
   static constexpr int kCount = kBatched + kSmall;
   static const char *name(int v) {
     static const char *n1[5] = {"32x8/352/3", "32x8/448/2", "32x16/640/2", "64x8/704/1", "32x8/352/2"};
     static const char *n2[2] = {"32x8/352/2", "32x8/448/2"};
     static const char *n16[2] = {"32x8/352/3", "32x8/352/2"};
     static const char *one1[3] = {"16x4/224/2", "32x4/384/2", "32x4/288/3"};
-    static const char *one2[2] = {"16x8/320/2", "32x4/384/1"};
+    static const char *one2[4] = {"32x12/480/1", "32x14/544/1", "16x8/320/2", "32x4/384/1"};
     if (v >= kBatched) return NH == 1 ? one1[v - kBatched] : one2[v - kBatched];
     return (FORM == 2 && NH == 1) ? n16[v] : (NH == 1 ? n1[v] : n2[v]);
   }
@@ -358,7 +358,9 @@ struct VariantTable {
         if (v == kBatched + 1) return launch_fused_t<32, 4, NH, FORM, 384, 2>(P, B, s);
         return launch_fused_t<32, 4, NH, FORM, 288, 3>(P, B, s);
       } else {
-        if (v == kBatched) return launch_fused_t<16, 8, NH, FORM, 320, 2>(P, B, s);
+        if (v == kBatched) return launch_fused_t<32, 12, NH, FORM, 480, 1>(P, B, s);
+        if (v == kBatched + 1) return launch_fused_t<32, 14, NH, FORM, 544, 1>(P, B, s);
+        if (v == kBatched + 2) return launch_fused_t<16, 8, NH, FORM, 320, 2>(P, B, s);
         return launch_fused_t<32, 4, NH, FORM, 384, 1>(P, B, s);
       }
     }
@@ -410,9 +412,11 @@ const char *fused_variant_name(const DevParams &P, int v) {
 //   180 x 360  32x8/448 7.4 us (270 tiles)      32x8/352/3 7.9  sweep 8.6 us
 //   200 x 400  sweep 8.1 us                     32x8/352/3 9.1 us (350 tiles, three to an SM)
 //   300 x 600  sweep 12.1 us                    32x8/352/3 14.4 us (750 tiles)
-// Three components: 128 x 128 16x8/320 5.3 us, 32x8/352 7.3, sweep 7.1; 100 x 200 16x8/320 6.6
-// us (175 tiles), 32x8/352 7.4; 256 x 256 32x8/352 9.4 us (256 tiles), 16x8/320 10.7 (512), sweep
-// 10.9; 512 x 512 sweep 22.0, 32x8/352 28.3 us.
+// Three components: 128 x 128 16x8/320 5.3 us, 32x8/352 7.3, sweep 7.1; 180 x 180 16x8/320 5.9
+// us (276 tiles), 32x8/352 6.8; then one large tile per SM, which recomputes less ring than two
+// small ones: 200 x 200 32x12/480 7.8 us (119 tiles), 32x8/352 8.8, sweep 8.1; 256 x 256
+// 32x14/544 8.7 us (152 tiles; C form 7.9), 32x8/352 8.9 (256 tiles; 8.3), sweep 10.3; 264 x 264
+// 32x8/352 8.9 us (297 tiles), sweep 10.4; 512 x 512 sweep 22.0, 32x8/352 28.3 us.
 int fused_default_variant(const DevParams &P) {
   static const int sms = [] {
     int dev = 0, n = 0;
@@ -429,7 +433,9 @@ int fused_default_variant(const DevParams &P) {
     if (tiles(32, 4) <= 3 * sms) return ns + nb + 2;
     if (tiles(32, 8) <= 2 * sms) return ns + 1;
   } else {
-    if (tiles(16, 8) <= 2 * sms) return ns + nb;
+    if (tiles(16, 8) <= 2 * sms) return ns + nb + 2;
+    if (tiles(32, 12) <= sms) return ns + nb;
+    if (tiles(32, 14) <= sms) return ns + nb + 1;
     if (tiles(32, 8) <= 2 * sms) return ns;
   }
   return sweep_default_variant(P, sms);
