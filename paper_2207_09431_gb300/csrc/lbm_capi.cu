@@ -236,7 +236,7 @@ lbm_status lbm_step(lbm_handle *h, long long nsteps) {
   cudaError_t e = cudaMemsetAsync(h->err, 0, sizeof(unsigned), h->stream);
   if (e != cudaSuccess) return h->cuda_fail(e, "lbm_step memset");
   long long t = 0;
-  // Runs of 16 and (small lattices) of 4 steps are replayed from captured graphs (on a
+  // Runs of 16 and of 4 steps are replayed from captured graphs (on a
   // created stream; capture needs one).  The last step writes the diagnostics and is
   // launched directly; a first run with a new configuration is too, so that
   // its kernels are configured outside the capture.  A graph starts from one of the two
@@ -245,13 +245,15 @@ lbm_status lbm_step(lbm_handle *h, long long nsteps) {
   // program of equal even runs captured anew on every call (64 steps of 64 x 128:
   // 333 -> 279 us, GB300).  A launch from the host takes some 6 us, longer than a step of a
   // lattice of up to about 150 x 300 nodes (3.6 to 6.4 us), whose last 15 steps therefore go
-  // in fours (279 -> 254 us); with larger ones the host is ahead of the device anyway.
+  // in fours (279 -> 254 us).  With larger ones the host is ahead of the device, and the fours
+  // save the wider gaps between direct launches, some 1.8 us each (64 steps of three
+  // components 256 x 256 604 -> 585 us); they are captured while the device is busy with the sixteens.
   const bool capturable = h->stream != nullptr && h->stream != cudaStreamLegacy && h->stream != cudaStreamPerThread;
   const bool small = (long long)h->prm.nx * h->prm.ny <= lbm_handle::kSmallNodes;
   for (auto &sg : h->graphs) {
-    if (!capturable || nsteps - 1 < sg.steps || (sg.steps < lbm_handle::kStepGraph && !small)) continue;
-    if (nsteps - 1 - t < sg.steps) continue;
     const bool captured = sg.exec && sg.variant == h->variant;
+    if (!capturable || nsteps - 1 - t < sg.steps) continue;
+    if (!captured && sg.steps < lbm_handle::kStepGraph && !small && t == 0) continue;
     if (captured ? sg.from != h->cur : t == 0) {
       h->launch_step(false, nullptr);
       ++t;

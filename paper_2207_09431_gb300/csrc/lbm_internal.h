@@ -214,7 +214,7 @@ struct lbm_handle {
     cudaGraphExec_t exec = nullptr;
   };
   static constexpr int kStepGraph = 16;
-  static constexpr long long kSmallNodes = 45000;  // lattices whose steps are shorter than a launch
+  static constexpr long long kSmallNodes = 45000;  // lattices whose step is shorter than a launch
   StepGraph graphs[2] = {{kStepGraph}, {4}};
   // lbm_set_fields: a stream of its own for the upload of C in row chunks,
   // overlapped with the conversion and initial equilibria on `stream`
