@@ -860,8 +860,9 @@ __global__ void __launch_bounds__(256) k_planes_to_f64(DevParams P, double3 rho,
     dst[o] = (double)c3;
     return;
   }
-  const double w1 = fmin(fmax((double)c1, 0.0), 1.0), w2 = fmin(fmax((double)c2, 0.0), 1.0),
-               w3 = fmin(fmax((double)c3, 0.0), 1.0);
+  // (by comparisons: fmin and fmax would turn a NaN into a weight of 0 and hide it)
+  auto clip = [](double v) { return v < 0.0 ? 0.0 : (v > 1.0 ? 1.0 : v); };
+  const double w1 = clip((double)c1), w2 = clip((double)c2), w3 = clip((double)c3);
   dst[o] = (w1 * rho.x + w2 * rho.y + w3 * rho.z) / (w1 + w2 + w3);
 }
 __global__ void __launch_bounds__(256) k_pops_to_f64(DevParams P, const float *__restrict__ src, int q0, int nq, int g16,
