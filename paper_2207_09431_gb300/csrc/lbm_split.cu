@@ -764,7 +764,7 @@ __global__ void __launch_bounds__(256) k_init(DevParams P, InitFields in, float 
       const float w = wt(a);
       const float eF = (n.mu[0] * n.dC[0][a] + n.mu[1] * n.dC[1][a] + n.mu[2] * n.dC[2][a]) +
                        (ex(a) * n.Fb[0] + ey(a) * n.Fb[1]);
-      ge[a] = -0.5f * (eF * w);
+      ge[a] = 0.0f - 0.5f * (eF * w);  // subtracted from w p = 0, as below: no force gives +0
       if constexpr (FORM == 0) {
 #pragma unroll
         for (int i = 0; i < NH; ++i) {
