@@ -35,3 +35,22 @@ def test_density_of_a_node_that_is_not_finite(lbm, ncomp, component, bad):
     got = lat.field("rho")
     assert np.array_equal(np.isnan(got), np.isnan(want)) and np.isnan(want).any() == np.isnan(bad)
     assert np.allclose(got, want, rtol=1e-14, atol=0, equal_nan=True)
+
+
+@pytest.mark.parametrize("rows", [5, 16, 17, 130])
+def test_gradients_with_a_weight_that_is_infinite(lbm, rows):
+    # a saturated unit (tanh = 1) leaves finite gradients, however many places of a 16-row tile are empty;
+    # tolerance of tests/test_gpu_surrogate.py
+    from oracle import mlp
+
+    w = inputs.mlp_init(1, seed=3)
+    w[0, 0] = np.inf
+    r = np.random.default_rng(rows)
+    X, T = np.abs(r.normal(size=(rows, 5))) + 0.1, r.normal(size=(rows, 2))
+    Y, loss, g = lbm.Surrogate(w, max_batch=rows, max_rows=rows).forward_backward(0, X, T)
+    params = inputs.mlp_unflatten(w[0])
+    Yo, cache = mlp.forward(params, X)
+    go = inputs.mlp_flatten(mlp.backward(params, cache, Yo, T))
+    assert np.isfinite(go).all() and np.isfinite(g).all() and np.isfinite(loss)
+    assert np.linalg.norm(Y - Yo) <= 1e-3 * np.linalg.norm(Yo)
+    assert np.linalg.norm(g - go) <= 1e-3 * np.linalg.norm(go)
