@@ -256,7 +256,8 @@ lbm_status lbm_batch_set_active(lbm_batch *b, int i, int active);
  * LBM_E_DIVERGED naming it in lbm_batch_last_error; the others advanced. */
 lbm_status lbm_batch_step(lbm_batch *b, long long nsteps);
 /* As lbm_autotune, over the whole work list; states are not advanced.  In
- * persistent mode only the sweep configurations are candidates. */
+ * persistent mode and with FP16 storage only the sweep configurations are
+ * candidates. */
 lbm_status lbm_batch_autotune(lbm_batch *b, int reps, int *chosen);
 /* Persistent mode (on = 1; 0 returns to one launch per step).  lbm_batch_step
  * then advances the whole ensemble in persistent cooperative launches of up to

@@ -366,8 +366,9 @@ lbm_status lbm_batch_autotune(lbm_batch *b, int reps, int *chosen) {
   if (!b || reps < 1) return LBM_E_INVAL;
   cudaError_t e = b->upload_table();
   if (e != cudaSuccess) return b->cuda_fail(e, "lbm_batch_autotune table");
-  // the persistent launch runs the sweep configurations only
-  const int nv = b->persistent ? lbm::sweep_batched_count(b->nh) : lbm::batched_variant_count(b->nh);
+  // the persistent launch and FP16 storage run the sweep configurations only
+  const bool sweeps = b->persistent || b->form == 2;
+  const int nv = sweeps ? lbm::sweep_batched_count(b->nh) : lbm::batched_variant_count(b->nh);
   cudaEvent_t e0, e1;
   if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess)
     return b->fail(LBM_E_CUDA, "cudaEventCreate");
