@@ -259,6 +259,11 @@ lbm_status lbm_batch_step(lbm_batch *b, long long nsteps);
  * persistent mode and with FP16 storage only the sweep configurations are
  * candidates. */
 lbm_status lbm_batch_autotune(lbm_batch *b, int reps, int *chosen);
+/* Number of launch configurations that lbm_batch_autotune chooses from in the
+ * batch's current mode, and explicit selection of one (for example the one it
+ * chose).  Every configuration computes the same values. */
+int lbm_batch_kernel_config_count(const lbm_batch *b);
+lbm_status lbm_batch_set_kernel_config(lbm_batch *b, int config);
 /* Persistent mode (on = 1; 0 returns to one launch per step).  lbm_batch_step
  * then advances the whole ensemble in persistent cooperative launches of up to
  * 4096 steps each (whole launches replayed from a captured CUDA graph on a

@@ -16,6 +16,7 @@
 
 #include "lbm.h"
 #include "lbm_internal.h"
+#include "lbm_schedule.h"
 
 namespace {
 
@@ -78,61 +79,6 @@ struct lbm_batch {
     for (auto *x : h) delete x;
   }
 
-  // Shared lists of a sweep: the strips of every running case laid end to end and cut
-  // into one share per CTA slot, shares equal in rows plus the pipeline fill of each
-  // piece (the smallest such size for which the slots suffice, by bisection).  A piece has
-  // at least kLeast rows and starts at a multiple of rs of its strip.  Piece k of share b stands at
-  // k * shares + b, empty pieces (y0 = y1) where a share has fewer.  Returns the shares, 0 if
-  // the padded list does not fit in cap.
-  static int share_out(const std::vector<lbm::WorkItem> &strips, int rs, int slots, size_t cap,
-                       std::vector<lbm::WorkItem> *out) {
-    constexpr int kLeast = 8;
-    const int fill = 3 * rs + rs * ((6 + rs - 1) / rs);
-    long long rows = 0;
-    int longest = 0;
-    for (const auto &s : strips) {
-      rows += s.y1;
-      longest = std::max(longest, s.y1);
-    }
-    // pieces of each share of `size` rows with their fills
-    auto cut = [&](long long size, std::vector<std::vector<lbm::WorkItem>> *shares) {
-      int used = 0;
-      long long left = 0;  // of the current share
-      for (const auto &s : strips) {
-        int y = 0;
-        while (y < s.y1) {
-          if (used == 0 || left - fill < std::min(kLeast, s.y1 - y)) {
-            ++used;
-            left = size;
-            if (shares) shares->emplace_back();
-          }
-          int len = (int)std::min<long long>(s.y1 - y, std::max<long long>(left - fill, kLeast));
-          if (len < s.y1 - y) len -= len % rs;
-          if (s.y1 - y - len < kLeast) len = s.y1 - y;  // no crumb for the next share
-          if (shares) shares->back().push_back({s.case_id, s.x0, y, y + len});
-          y += len;
-          left -= len + fill;
-        }
-      }
-      return used;
-    };
-    long long lo = 1, hi = rows + (long long)fill * (long long)strips.size() + fill + kLeast;  // hi: one share
-    while (lo < hi) {
-      const long long mid = (lo + hi) / 2;
-      if (cut(mid, nullptr) <= slots) hi = mid;
-      else lo = mid + 1;
-    }
-    std::vector<std::vector<lbm::WorkItem>> shares;
-    const int n = cut(hi, &shares);
-    size_t deepest = 0;
-    for (const auto &s : shares) deepest = std::max(deepest, s.size());
-    if (n > slots || deepest * (size_t)n > cap) return 0;
-    out->assign(deepest * (size_t)n, lbm::WorkItem{0, 0, 0, 0});
-    for (int b = 0; b < n; ++b)
-      for (size_t k = 0; k < shares[b].size(); ++k) (*out)[k * (size_t)n + b] = shares[b][k];
-    return n;
-  }
-
   // Work list of the active, initialised cases for configuration v (tiles, strips x
   // row segments, or shared lists of a sweep); uploads it.  *ctas: the CTAs that share
   // it, 0 for one item per CTA.
@@ -152,7 +98,7 @@ struct lbm_batch {
       int slots = 0;
       const cudaError_t e = lbm::sweep_batched_slots(nh, form, v, persistent, &slots);
       if (e != cudaSuccess) return e;
-      if (!strips.empty()) *ctas = share_out(strips, rs, slots, work_cap, &w);
+      if (!strips.empty()) *ctas = lbm::share_out(strips, rs, slots, work_cap, &w);
       if (*ctas == 0) ty = 96;  // no room for the lists: segments
     }
     if (*ctas == 0) {
@@ -366,9 +312,7 @@ lbm_status lbm_batch_autotune(lbm_batch *b, int reps, int *chosen) {
   if (!b || reps < 1) return LBM_E_INVAL;
   cudaError_t e = b->upload_table();
   if (e != cudaSuccess) return b->cuda_fail(e, "lbm_batch_autotune table");
-  // the persistent launch and FP16 storage run the sweep configurations only
-  const bool sweeps = b->persistent || b->form == 2;
-  const int nv = sweeps ? lbm::sweep_batched_count(b->nh) : lbm::batched_variant_count(b->nh);
+  const int nv = lbm_batch_kernel_config_count(b);
   cudaEvent_t e0, e1;
   if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess)
     return b->fail(LBM_E_CUDA, "cudaEventCreate");
@@ -399,6 +343,21 @@ lbm_status lbm_batch_autotune(lbm_batch *b, int reps, int *chosen) {
   b->variant = best;
   b->work_valid = false;
   if (chosen) *chosen = best;
+  return LBM_OK;
+}
+
+int lbm_batch_kernel_config_count(const lbm_batch *b) {
+  if (!b) return 0;
+  // the persistent launch and FP16 storage run the sweep configurations only
+  return b->persistent || b->form == 2 ? lbm::sweep_batched_count(b->nh) : lbm::batched_variant_count(b->nh);
+}
+
+lbm_status lbm_batch_set_kernel_config(lbm_batch *b, int config) {
+  if (!b) return LBM_E_INVAL;
+  if (config < 0 || config >= lbm_batch_kernel_config_count(b))
+    return b->fail(LBM_E_INVAL, "no such kernel configuration");
+  b->variant = config;
+  b->work_valid = false;
   return LBM_OK;
 }
 

@@ -78,7 +78,8 @@ EXPORTED = ["lbm_version", "lbm_required_bytes", "lbm_create", "lbm_init_bubbles
             "lbm_profile_step", "lbm_observables_static", "lbm_autotune", "lbm_kernel_config_count",
             "lbm_set_kernel_config", "lbm_batch_required_bytes", "lbm_batch_create", "lbm_batch_case",
             "lbm_batch_set_active", "lbm_batch_step", "lbm_batch_autotune", "lbm_batch_destroy",
-            "lbm_batch_last_error", "lbm_batch_set_persistent", "lbm_batch_run", "surr_param_count", "surr_required_bytes", "surr_create", "surr_destroy",
+            "lbm_batch_last_error", "lbm_batch_set_persistent", "lbm_batch_run", "lbm_batch_kernel_config_count",
+            "lbm_batch_set_kernel_config", "surr_param_count", "surr_required_bytes", "surr_create", "surr_destroy",
             "surr_last_error", "surr_get_weights", "surr_forward_backward", "surr_train", "surr_predict", "surr_answer",
             "surr_train_cv", "surr_local_residual", "surr_set_local_trust"]
 
@@ -125,6 +126,8 @@ def load_library(path: str | None = None):
     lib.lbm_batch_set_active.argtypes = [vp, ctypes.c_int, ctypes.c_int]
     lib.lbm_batch_step.argtypes = [vp, ctypes.c_longlong]
     lib.lbm_batch_autotune.argtypes = [vp, ctypes.c_int, P(ctypes.c_int)]
+    lib.lbm_batch_kernel_config_count.argtypes = [vp]
+    lib.lbm_batch_set_kernel_config.argtypes = [vp, ctypes.c_int]
     lib.lbm_batch_set_persistent.argtypes = [vp, ctypes.c_int, ctypes.c_longlong]
     lib.lbm_batch_run.argtypes = [vp, P(lbm_run_opts), P(lbm_obs), P(ctypes.c_int), P(ctypes.c_longlong)]
     lib.lbm_batch_destroy.argtypes = [vp]
@@ -362,6 +365,14 @@ def lbm_batch_autotune(b, reps: int = 3) -> int:
     chosen = ctypes.c_int(0)
     _check_batch(b, load_library().lbm_batch_autotune(b, int(reps), ctypes.byref(chosen)), "lbm_batch_autotune")
     return int(chosen.value)
+
+
+def lbm_batch_kernel_config_count(b) -> int:
+    return load_library().lbm_batch_kernel_config_count(b)
+
+
+def lbm_batch_set_kernel_config(b, config: int):
+    _check_batch(b, load_library().lbm_batch_set_kernel_config(b, int(config)), "lbm_batch_set_kernel_config")
 
 
 def lbm_batch_set_persistent(b, on: bool = True, spin_limit: int = 0):
