@@ -199,9 +199,10 @@ void lbm_destroy(lbm_handle *h);
 int lbm_kernels_per_step(const lbm_handle *h);
 const char *lbm_kernel_name(const lbm_handle *h, int i);
 
-/* Times each launch configuration of the fused step (tile shape, threads per
- * CTA, CTAs per SM) for `reps` launches from the current state into the spare
- * buffer, without advancing the state, and keeps the fastest for lbm_step.
+/* Times the launch configurations of the fused step (tile shape, threads per
+ * CTA, CTAs per SM) that suit the lattice's size for `reps` launches from the
+ * current state into the spare buffer, without advancing the state, and keeps
+ * the fastest for lbm_step.
  * chosen (may be NULL) receives its index; lbm_kernel_name reports its name.
  * Synchronises the stream.  A handle starts with the configuration that
  * measured fastest on lattices of its size (its name through lbm_kernel_name). */

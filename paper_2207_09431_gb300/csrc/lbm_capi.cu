@@ -548,10 +548,11 @@ lbm_status lbm_autotune(lbm_handle *h, int reps, int *chosen) {
   // every candidate runs from the current state into the spare buffer; the
   // state itself is not advanced
   const lbm::FusedBuffers B = h->fused_buffers(h->cur, false);
-  int best = 0;
+  int best = -1;
   float best_ms = 0.f;
   cudaError_t err = cudaSuccess;
   for (int v = 0; v < nv && err == cudaSuccess; ++v) {
+    if (!lbm::fused_variant_timed(h->dp, v)) continue;
     err = lbm::launch_fused_step(h->dp, B, h->stream, v);  // warm-up and attribute set-up
     if (err != cudaSuccess) break;
     cudaEventRecord(e0, h->stream);
@@ -560,7 +561,7 @@ lbm_status lbm_autotune(lbm_handle *h, int reps, int *chosen) {
     err = cudaEventSynchronize(e1);
     float ms = 0.f;
     if (err == cudaSuccess) err = cudaEventElapsedTime(&ms, e0, e1);
-    if (err == cudaSuccess && (v == 0 || ms < best_ms)) {
+    if (err == cudaSuccess && (best < 0 || ms < best_ms)) {
       best = v;
       best_ms = ms;
     }

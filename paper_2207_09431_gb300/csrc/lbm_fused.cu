@@ -417,7 +417,7 @@ const char *fused_variant_name(const DevParams &P, int v) {
 // small ones: 200 x 200 32x12/480 7.8 us (119 tiles), 32x8/352 8.8, sweep 8.1; 256 x 256
 // 32x14/544 8.7 us (152 tiles; C form 7.9), 32x8/352 8.9 (256 tiles; 8.3), sweep 10.3; 264 x 264
 // 32x8/352 8.9 us (297 tiles), sweep 10.4; 512 x 512 sweep 22.0, 32x8/352 28.3 us.
-int fused_default_variant(const DevParams &P) {
+static int device_sms() {
   static const int sms = [] {
     int dev = 0, n = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
@@ -425,8 +425,17 @@ int fused_default_variant(const DevParams &P) {
       return 152;
     return n;
   }();
-  auto tiles = [&](int tx, int ty) { return (long long)((P.nx + tx - 1) / tx) * ((P.ny + ty - 1) / ty); };
-  const int ns = sweep_variant_count(P), nb = form_of(P) == 2 || P.nh == 2 ? 2 : 5;
+  return sms;
+}
+static long long tiles_of(const DevParams &P, int tx, int ty) {
+  return (long long)((P.nx + tx - 1) / tx) * ((P.ny + ty - 1) / ty);
+}
+static int batched_tiles(const DevParams &P) { return form_of(P) == 2 || P.nh == 2 ? 2 : 5; }
+
+int fused_default_variant(const DevParams &P) {
+  const int sms = device_sms();
+  auto tiles = [&](int tx, int ty) { return tiles_of(P, tx, ty); };
+  const int ns = sweep_variant_count(P), nb = batched_tiles(P);
   if (P.nh == 1) {
     if (tiles(16, 4) <= sms) return ns + nb;
     if (tiles(32, 4) <= 2 * sms) return ns + nb + 1;
@@ -439,6 +448,25 @@ int fused_default_variant(const DevParams &P) {
     if (tiles(32, 8) <= 2 * sms) return ns;
   }
   return sweep_default_variant(P, sms);
+}
+
+// Whether the autotuner times configuration v: all but those that the lattice's size rules
+// out.  A tile for small lattices is timed where the device holds all of them at once; past that
+// it ran up to twice as long as the best (three components 1024 x 1024: four such tiles
+// took as long as the six others).  A sweep is not timed on lattices of one wave of the smallest
+// tiles, 16 x 4 or 16 x 8: over such lattices from 3 x 3 to 4000 x 8 and 16 x 2400, in every state
+// form, the best sweep took 1.13 to 1.72 times the tile's time (64 x 128 5.5 against 3.8 us).
+// lbm_autotune of 2 repetitions without this rule and with it: 64 x 40 710 and 267 us, 1024 x 1024
+// 4544 and 3461 us, three components 1024 x 1024 3630 and 1763 us (GB300).
+bool fused_variant_timed(const DevParams &P, int v) {
+  const int sms = device_sms(), ns = sweep_variant_count(P), nb = batched_tiles(P);
+  if (v < ns) return P.nh == 1 ? tiles_of(P, 16, 4) > sms : tiles_of(P, 16, 8) > 2 * sms;
+  if (v < ns + nb) return true;
+  // tile and CTAs per SM, in the order of VariantTable
+  static const int one1[3][3] = {{16, 4, 2}, {32, 4, 2}, {32, 4, 3}};
+  static const int one2[4][3] = {{32, 12, 1}, {32, 14, 1}, {16, 8, 2}, {32, 4, 1}};
+  const int *t = P.nh == 1 ? one1[v - ns - nb] : one2[v - ns - nb];
+  return tiles_of(P, t[0], t[1]) <= (long long)t[2] * sms;
 }
 
 cudaError_t launch_fused_step(const DevParams &P, const FusedBuffers &B, cudaStream_t s, int v) {

@@ -96,6 +96,8 @@ const char *sweep_variant_name(const DevParams &P, int v);
 // Configuration a handle starts with, by the lattice size (sweep: of those only).
 int sweep_default_variant(const DevParams &P, int sms);
 int fused_default_variant(const DevParams &P);
+// Whether the autotuner times configuration v on a lattice of this size.
+bool fused_variant_timed(const DevParams &P, int v);
 cudaError_t launch_sweep_step(const DevParams &P, const FusedBuffers &B, cudaStream_t s, int v);
 int fused_variant_count(const DevParams &P);
 const char *fused_variant_name(const DevParams &P, int v);
