@@ -806,12 +806,16 @@ struct BatchedSweep {
 // their columns empty there), in the C form 291 against 269 us (60 columns; the larger record
 // of that form leaves one CTA of the 100-column strips per SM); 48 cases of 100 x 200 to 300 x
 // 600 196 against 187 us, C form 204 against 194 us.  Shares of 58 columns were no better than
-// those of 60, nor four-row strips of 50.
-static const int kShapes1[12][2] = {{58, 48}, {58, 96},  {60, 48},  {64, 48},  {58, 64}, {58, 72},
-                                    {60, 64}, {60, 128}, {60, 200}, {58, 160}, {60, 0},  {100, 0}};
-static const int kShapes2[4][2] = {{64, 48}, {62, 48}, {64, 0}, {62, 0}};
+// those of 60, nor four-row strips of 50.  Every shape in the list costs a lbm_batch_autotune two
+// launches and more: over 46 ensembles of 1 to 256 cases, in each form and mode, leaving out
+// segments of 64, 96 and 160 rows (58 columns), 64 and 200 (60 columns) and, with three components, all
+// segments cost at most 0.1 % (three components 1.1 %) of the step and nothing on most.
+// lbm_batch_autotune of one repetition with them and now, 256 cases of 100 x 200: 15.0 and 11.8 ms,
+// persistent 7.4 and 4.3 ms, three components 8.0 and 6.0 ms (GB300).
+static const int kShapes1[7][2] = {{58, 48}, {60, 48}, {64, 48}, {58, 72}, {60, 128}, {60, 0}, {100, 0}};
+static const int kShapes2[2][2] = {{64, 0}, {62, 0}};
 
-int sweep_batched_count(int nh) { return nh == 1 ? 12 : 4; }
+int sweep_batched_count(int nh) { return nh == 1 ? 7 : 2; }
 
 void sweep_batched_shape(int nh, int v, int *tx, int *rows) {
   if (v < 0 || v >= sweep_batched_count(nh)) v = 0;

@@ -57,7 +57,7 @@ def test_every_configuration_equals_single_lattices(lbm, shapes, form, persisten
     batch = lbm.Batch([p for p, _, _ in cases])
     batch.set_persistent(persistent)
     count = lbm.lbm_batch_kernel_config_count(batch.b)
-    assert count >= 4
+    assert count >= 2
     for config in range(count):
         for i, (_, C, u) in enumerate(cases):
             batch.case(i).set_fields(C, ux=u, uy=-u)
