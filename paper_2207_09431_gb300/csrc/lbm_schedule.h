@@ -7,6 +7,35 @@
 
 namespace lbm {
 
+// Segment length for a strip count: the number of segments per strip that
+// minimises the rows the slowest CTA sweeps, waves x (segment rows + the
+// pipeline fill of fill rows), with the rows of a strip split evenly (a multiple of
+// rs each, the last segment the shortest); the fewest segments among equals.  Segments are the
+// shorter the more of them a number of waves holds, so one candidate per number of waves
+// is enough, up to the waves of which the fills alone cost as much as the best.  Every launch asks
+// for it, and lbm_create for up to seven shapes.  With a walk over every number of segments
+// lbm_create took 269 us at 2048 x 4096 and 711 us at 1 x 50000, with this one 217 and 53 us (GB300,
+// Grace host; 215 and 51 us of it clear the arena).
+inline int choose_segment(int ny, int strips, int resident, int rs, int fill) {
+  int best_len = ny;
+  long long best_cost = -1;
+  const long long most = (ny + rs - 1) / rs;  // segments
+  for (long long waves = (strips + resident - 1) / resident; best_cost < 0 || waves * (rs + fill) < best_cost; ++waves) {
+    const long long nseg = std::min(most, waves * resident / strips);
+    int len = (int)((ny + nseg - 1) / nseg);
+    len = (len + rs - 1) / rs * rs;
+    // (rounding the length up may leave fewer segments, and waves)
+    const long long total = (ny + len - 1) / len * (long long)strips;
+    const long long cost = (total + resident - 1) / resident * (len + fill);
+    if (best_cost < 0 || cost < best_cost) {
+      best_cost = cost;
+      best_len = len;
+    }
+    if (nseg == most) break;
+  }
+  return best_len;
+}
+
 // Shared lists of a sweep: the strips of every running case laid end to end and cut
 // into one share per CTA slot, shares equal in rows plus the pipeline fill of each
 // piece (the smallest such size for which the slots suffice, by bisection).  Item is

@@ -34,6 +34,7 @@
 
 #include "lbm_kernels.h"
 #include "lbm_node.cuh"
+#include "lbm_schedule.h"
 
 namespace lbm {
 
@@ -587,28 +588,6 @@ __global__ void __launch_bounds__(NT, MINB) k_sweep_persistent(const BatchCase *
     }
     if (t + 1 < nsteps && !grid_barrier(sync, gridDim.x, spin_limit)) return;
   }
-}
-
-// Segment length for a strip count: the number of segments per strip that
-// minimises the rows the slowest CTA sweeps, waves x (segment rows + the
-// pipeline fill of fill rows), with the rows of a strip split evenly (a multiple of
-// rs each, the last segment the shortest).
-int choose_segment(int ny, int strips, int resident, int rs, int fill) {
-  int best_len = ny;
-  long long best_cost = -1;
-  for (int nseg = 1; nseg <= (ny + rs - 1) / rs; ++nseg) {
-    int len = (ny + nseg - 1) / nseg;
-    len = (len + rs - 1) / rs * rs;
-    if ((ny + len - 1) / len != nseg) continue;  // rounding merged two segments
-    const long long total = (long long)strips * nseg;
-    const long long waves = (total + resident - 1) / resident;
-    const long long cost = waves * (len + fill);
-    if (best_cost < 0 || cost < best_cost) {
-      best_cost = cost;
-      best_len = len;
-    }
-  }
-  return best_len;
 }
 
 template <int TX, int RS, int NH, int FORM, int PER, int NT, int MINB>

@@ -1,5 +1,6 @@
 """The host arithmetic that splits the rows of sweeps over the CTAs (csrc/lbm_schedule.h), built with the
-host compiler: shared lists of a batch hold every row of every strip once, whatever the cases."""
+host compiler: shared lists of a batch hold every row of every strip once, whatever the cases, and segment
+lengths are those of a search over every number of segments."""
 import os
 import random
 import subprocess
@@ -13,7 +14,14 @@ MAIN = r"""
 #include "lbm_schedule.h"
 struct Item { int case_id, x0, y0, y1; };
 // reads "rs slots cap strips", then the rows of each strip; prints the shares and their items
-int main() {
+// with an argument: "ny strips resident rs fill", prints the segment length
+int main(int argc, char **) {
+  if (argc > 1) {
+    int ny, strips, resident, step, fill;
+    while (std::scanf("%d %d %d %d %d", &ny, &strips, &resident, &step, &fill) == 5)
+      std::printf("%d\n", lbm::choose_segment(ny, strips, resident, step, fill));
+    return 0;
+  }
   int rs, slots, n;
   unsigned long long cap;
   while (std::scanf("%d %d %llu %d", &rs, &slots, &cap, &n) == 4) {
@@ -40,7 +48,11 @@ def run(tmp_path_factory):
     subprocess.run(["g++", "-std=c++17", "-O1", "-Wall", "-Werror", "-I", CSRC, str(d / "main.cpp"), "-o", str(d / "main")],
                    check=True)
 
-    def call(queries):
+    def call(queries, *arguments):
+        if arguments:
+            text = "\n".join(" ".join(map(str, q)) for q in queries)
+            out = subprocess.run([str(d / "main"), *arguments], input=text, capture_output=True, text=True, check=True)
+            return [int(line) for line in out.stdout.splitlines()]
         text = "\n".join(" ".join(map(str, (rs, slots, cap, len(rows), *rows))) for rs, slots, cap, rows in queries)
         out = subprocess.run([str(d / "main")], input=text, capture_output=True, text=True, check=True).stdout
         return [list(map(int, line.split())) for line in out.splitlines()]
@@ -92,3 +104,27 @@ def test_shared_lists_hold_every_row_once(run):
 
 def test_lists_that_do_not_fit_are_refused(run):
     assert run([(2, 1, 2, [20, 20, 20])]) == [[0, 0]]
+
+
+def segment(ny, strips, resident, rs, fill):
+    best = None
+    for nseg in range(1, -(-ny // rs) + 1):
+        length = -(-(-(-ny // nseg)) // rs) * rs
+        if -(-ny // length) != nseg:
+            continue  # rounding merged two segments
+        cost = -(-strips * nseg // resident) * (length + fill)
+        if best is None or cost < best[0]:
+            best = cost, length
+    return best[1] if best else ny
+
+
+def test_segment_length_is_the_best_of_all(run):
+    r = random.Random(9)
+    asked = []
+    for _ in range(4000):
+        rs = r.choice((1, 2, 3, 4, 6, 8))
+        ny = r.choice((r.randint(3, 40), r.randint(3, 700), r.randint(3, 3000)))
+        strips = r.choice((1, r.randint(1, 40), r.randint(1, 3000)))
+        asked.append((ny, strips, r.choice((152, 304, 456, 760, r.randint(1, 50))), rs, 3 * rs + rs * -(-6 // rs)))
+    for q, got in zip(asked, run(asked, "segments")):
+        assert got == segment(*q), q
