@@ -103,11 +103,25 @@ lbm_status lbm_create(const lbm_params *p, void *dev_arena, size_t arena_bytes, 
   return LBM_OK;
 }
 
-// Whether lbm_set_fields may overlap the upload with the initial equilibria: chunks
-// of at least 16 rows (the equilibria read two rows beyond their own), and a stream
-// that is not being captured.  The copy stream and its events are created on first use.
-static bool upload_overlappable(lbm_handle *h) {
+// Whether lbm_set_fields overlaps the upload with the initial equilibria: C of 32 MB and more in
+// page-locked memory, as the other fields, chunks of at least 16 rows (the equilibria read two rows
+// beyond their own), and a stream that is not being captured.  A copy from pageable memory returns when it
+// is done, and 4 to 16 small copies, events and launches cost more than they hide in smaller
+// fields.  Whole and in chunks, us (GB300): C pageable 200 x 400 30 and 72, 2048 x 4096 547 and 601;
+// C, p and u pageable 200 x 400 75 and 203; C page-locked 200 x 400 22 and 35, 1024 x 2048 135 and
+// 133, 2048 x 4096 467 and 419.  The copy stream and its events are created on first use.
+static bool upload_overlappable(lbm_handle *h, const double *C, const double *const f[3]) {
   if (h->prm.ny < 16 * lbm_handle::kUploadChunks) return false;
+  if ((size_t)(h->prm.ncomp - 1) * h->prm.nx * h->prm.ny * sizeof(double) < ((size_t)32 << 20)) return false;
+  for (const double *p : {C, f[0], f[1], f[2]}) {
+    cudaPointerAttributes a{};
+    if (!p) continue;
+    if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+      cudaGetLastError();  // not CUDA's memory: nothing else asks for this error
+      return false;
+    }
+    if (a.type != cudaMemoryTypeHost) return false;
+  }
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
   if (cudaStreamIsCapturing(h->stream, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) return false;
   if (!h->copy_stream && cudaStreamCreateWithFlags(&h->copy_stream, cudaStreamNonBlocking) != cudaSuccess) {
@@ -192,7 +206,7 @@ lbm_status lbm_set_fields(lbm_handle *h, const double *C, const double *p, const
   const StagedFields st(h);
   const double *const f[3] = {p, ux, uy};
   const bool given[3] = {p != nullptr, ux != nullptr, uy != nullptr};
-  if (upload_overlappable(h)) return fields_set(h, upload_and_init_overlapped(h, st, C, f, given));
+  if (upload_overlappable(h, C, f)) return fields_set(h, upload_and_init_overlapped(h, st, C, f, given));
   const size_t bytes = (size_t)h->prm.nx * h->prm.ny * sizeof(double);
   cudaError_t e = cudaMemcpyAsync(st.C, C, nh * bytes, cudaMemcpyHostToDevice, h->stream);
   for (int q = 0; q < 3 && e == cudaSuccess; ++q)

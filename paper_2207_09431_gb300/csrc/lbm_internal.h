@@ -216,8 +216,8 @@ struct lbm_handle {
   static constexpr int kStepGraph = 16;
   static constexpr long long kSmallNodes = 45000;  // lattices whose step is shorter than a launch
   StepGraph graphs[2] = {{kStepGraph}, {4}};
-  // lbm_set_fields: a stream of its own for the upload of C in row chunks,
-  // overlapped with the conversion and initial equilibria on `stream`
+  // lbm_set_fields: a stream of its own for the upload of large page-locked fields in
+  // row chunks, overlapped with the initial equilibria on `stream`
   static constexpr int kUploadChunks = 4;
   cudaStream_t copy_stream = nullptr;
   cudaEvent_t upload_ev[kUploadChunks + 1] = {};
