@@ -33,11 +33,32 @@ static void map_pages(double *dst, size_t values) {
   }
 }
 
+// Small fields are converted on the host from the FP32 planes as they are stored: planes of up to
+// 8192 floats together, populations of up to 2560 nodes in planes of up to 4096.  Above, the loop costs more than a launch and twice the
+// bytes; below, us per lbm_get_field on the host and on the device (GB300, Grace host): tau 64 x 40
+// 15.4 and 18.6, 64 x 128 16.8 and 19.1, 100 x 200 18.2 and 19.4 but u_x 34.8 and 33.0; g 16 x 16 17
+// and 43, 64 x 40 43 and 45, 60 x 60 51 and 46.
+constexpr size_t kHostPlanes = 8192, kHostPopulations = 2560;
+static cudaError_t staged_on_host(lbm_handle *h, const float *src, size_t floats) {
+  h->stage.resize(floats);
+  const cudaError_t e = cudaMemcpyAsync(h->stage.data(), src, floats * sizeof(float), cudaMemcpyDeviceToHost, h->stream);
+  return e == cudaSuccess ? cudaStreamSynchronize(h->stream) : e;
+}
+
 // Fields go to the host as dense doubles, converted on the device in the spare
 // population buffer (free between steps; four dense planes of doubles fit) and copied
 // straight into the caller's array.
 static cudaError_t download_planes(lbm_handle *h, const float *src, double *dst, int nplanes, int kind = lbm::kPlane) {
   const size_t N = (size_t)h->prm.nx * h->prm.ny;
+  if (kind == lbm::kPlane && nplanes * h->plane_floats() <= kHostPlanes) {
+    cudaError_t e = staged_on_host(h, src, nplanes * h->plane_floats());
+    for (int q = 0; q < nplanes && e == cudaSuccess; ++q)
+      for (int y = 0; y < h->prm.ny; ++y) {
+        const float *row = h->stage.data() + q * h->plane_floats() + (size_t)y * h->dp.pitch;
+        std::copy(row, row + h->prm.nx, dst + (q * (size_t)h->prm.ny + y) * h->prm.nx);
+      }
+    return e;
+  }
   double *dense = reinterpret_cast<double *>(h->g[1 - h->cur]);
   cudaError_t e = lbm::launch_planes_to_f64(h->dp, h->prm.rho, src, kind, nplanes, dense, h->stream);
   map_pages(dst, nplanes * N);
@@ -50,6 +71,14 @@ static cudaError_t download_planes(lbm_handle *h, const float *src, double *dst,
 // The nq planes of a device population array, plane after plane.
 static cudaError_t download_pops(lbm_handle *h, const float *src, double *dst, int nq, bool g16) {
   const size_t N = (size_t)h->prm.nx * h->prm.ny;
+  if (!g16 && N <= kHostPopulations && h->plane_floats() <= 4096) {
+    cudaError_t e = staged_on_host(h, src, nq * h->plane_floats());
+    for (int q = 0; q < nq && e == cudaSuccess; ++q)
+      for (int y = 0; y < h->prm.ny; ++y)
+        for (int x = 0; x < h->prm.nx; ++x)
+          *dst++ = h->stage[lbm::pop_index((long long)y * h->dp.pitch + x, q, nq)];
+    return e;
+  }
   double *dense = reinterpret_cast<double *>(h->g[1 - h->cur]);
   cudaError_t e = cudaSuccess;
   for (int q0 = 0; q0 < nq && e == cudaSuccess; q0 += 4) {

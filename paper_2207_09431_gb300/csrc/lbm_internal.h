@@ -207,6 +207,7 @@ struct lbm_handle {
   long long prev_step;
   double prev_v, y_int;
   std::string last_error;
+  std::vector<float> stage;  // a small field as stored, on its way to the host's doubles
   // captured runs of steps without diagnostics, each for the starting buffer (cur)
   // and the launch configuration it was captured with
   struct StepGraph {

@@ -46,3 +46,27 @@ def test_new_memory_is_filled_and_nothing_else(lbm, nx, ny, form):
             assert values[before + want.size] == -8.5 and (not before or values[before - 1] == -7.5)
             assert not values[before + want.size + 1:].any() and not values[:max(0, before - 1)].any()
             del values, array
+
+
+@pytest.mark.parametrize("nx,ny", [(8, 320), (8, 321), (64, 40), (41, 64), (64, 64), (64, 65), (128, 64), (91, 91)])
+@pytest.mark.parametrize("ncomp", [2, 3])
+def test_small_fields_equal_the_stored_state(lbm, nx, ny, ncomp):
+    """Either side of the sizes that are converted on the host, against the arena's own planes (include/lbm.h)."""
+    p, _ = inputs.small_case(mobility=1)
+    p = dict(p, nx=nx, ny=ny, ncomp=ncomp)
+    lat = lbm.Lattice(p)
+    lat.set_fields(inputs.bubble_fields(nx, ny, ncomp, p["xi"], [(nx / 2, ny / 3, 3.0, 3)], seed=1, noise=1e-4))
+    pitch, nh = (nx + 31) // 32 * 32, ncomp - 1
+    plane = (ny * pitch * 4 + 255) // 256 * 64
+    for steps in (0, 2):  # buffer 0 holds the state after an even number of steps
+        lat.step(steps)
+        words = lat.arena.cpu().numpy().view(np.float32)
+
+        def populations(first, nq):
+            v = words[first:first + nq * ny * pitch].reshape(ny, pitch // 32, nq, 32)
+            return v.transpose(2, 0, 1, 3).reshape(nq, ny, pitch)[:, :, :nx].astype(np.float64)
+
+        assert np.array_equal(lat.field("g"), populations(0, 9))
+        assert np.array_equal(lat.field("h").reshape(9 * nh, ny, nx), populations(18 * plane, 9 * nh))
+        tau = words[(18 + 18 * nh) * plane:][:ny * pitch].reshape(ny, pitch)[:, :nx]
+        assert np.array_equal(lat.field("tau"), tau.astype(np.float64))
