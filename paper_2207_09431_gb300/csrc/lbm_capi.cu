@@ -309,12 +309,19 @@ lbm_status lbm_step(lbm_handle *h, long long nsteps) {
   // in fours (279 -> 254 us).  With larger ones the host is ahead of the device, and the fours
   // save the wider gaps between direct launches, some 1.8 us each (64 steps of three
   // components 256 x 256 604 -> 585 us); they are captured while the device is busy with the sixteens.
+  // Without sixteens before them a capture costs as much as the launches of two runs, so a handle
+  // captures the fours on its second missed run (first call of a new handle of 64 x 128, 5 and 8 steps:
+  // 64 and 77 us with a capture, 52 and 69 without).
   const bool capturable = h->stream != nullptr && h->stream != cudaStreamLegacy && h->stream != cudaStreamPerThread;
   const bool small = (long long)h->prm.nx * h->prm.ny <= lbm_handle::kSmallNodes;
   for (auto &sg : h->graphs) {
     const bool captured = sg.exec && sg.variant == h->variant;
     if (!capturable || nsteps - 1 - t < sg.steps) continue;
-    if (!captured && sg.steps < lbm_handle::kStepGraph && !small && t == 0) continue;
+    if (!captured && sg.steps < lbm_handle::kStepGraph && t == 0) {
+      if (!small) continue;
+      sg.missed += (int)std::min<long long>((nsteps - 1) / sg.steps, 2);
+      if (sg.missed < 2) continue;
+    }
     if (captured ? sg.from != h->cur : t == 0) {
       h->launch_step(false, nullptr);
       ++t;
@@ -340,6 +347,7 @@ lbm_status lbm_step(lbm_handle *h, long long nsteps) {
       }
       sg.variant = h->variant;
       sg.from = c;
+      sg.missed = 0;
     }
     for (; nsteps - 1 - t >= sg.steps && e == cudaSuccess; t += sg.steps) e = cudaGraphLaunch(sg.exec, h->stream);
     if (e != cudaSuccess) return h->cuda_fail(e, "lbm_step graph launch");

@@ -212,6 +212,7 @@ struct lbm_handle {
   // and the launch configuration it was captured with
   struct StepGraph {
     int steps, variant = -1, from = -1;
+    int missed = 0;  // runs of this length launched directly since the last capture (up to a few)
     cudaGraphExec_t exec = nullptr;
   };
   static constexpr int kStepGraph = 16;
