@@ -786,15 +786,17 @@ struct BatchedSweep {
 // of that form leaves one CTA of the 100-column strips per SM); 48 cases of 100 x 200 to 300 x
 // 600 196 against 187 us, C form 204 against 194 us.  Shares of 58 columns were no better than
 // those of 60, nor four-row strips of 50.  Every shape in the list costs a lbm_batch_autotune two
-// launches and more: over 46 ensembles of 1 to 256 cases, in each form and mode, leaving out
-// segments of 64, 96 and 160 rows (58 columns), 64 and 200 (60 columns) and, with three components, all
-// segments cost at most 0.1 % (three components 1.1 %) of the step and nothing on most.
-// lbm_batch_autotune of one repetition with them and now, 256 cases of 100 x 200: 15.0 and 11.8 ms,
-// persistent 7.4 and 4.3 ms, three components 8.0 and 6.0 ms (GB300).
-static const int kShapes1[7][2] = {{58, 48}, {60, 48}, {64, 48}, {58, 72}, {60, 128}, {60, 0}, {100, 0}};
-static const int kShapes2[2][2] = {{64, 0}, {62, 0}};
+// launches and more.  Segments of 64, 96 and 160 rows (58 columns), and with three components of 48
+// rows (64 columns), are not in it: over 80 ensembles of 1 to 1024 cases in each form and mode the best of
+// the others is within 0.1 % of theirs.  Each of the rest is the best by 1 to 6 % for some, such as the
+// 200-row segments for 128 cases of the default grids in the C form (2 to 4 %).  lbm_batch_autotune
+// of one repetition with all twelve (four) and with these, 256 cases of 100 x 200: 15.0 and 13.2 ms, persistent
+// 7.4 and 5.6 ms, three components 8.0 and 6.9 ms (GB300; before the shared lists 13.9, 6.3 and 6.1 ms).
+static const int kShapes1[9][2] = {{58, 48}, {60, 48},  {64, 48},  {58, 72}, {60, 64},
+                                   {60, 128}, {60, 200}, {60, 0}, {100, 0}};
+static const int kShapes2[3][2] = {{64, 0}, {62, 0}, {62, 48}};
 
-int sweep_batched_count(int nh) { return nh == 1 ? 7 : 2; }
+int sweep_batched_count(int nh) { return nh == 1 ? 9 : 3; }
 
 void sweep_batched_shape(int nh, int v, int *tx, int *rows) {
   if (v < 0 || v >= sweep_batched_count(nh)) v = 0;
