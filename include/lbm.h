@@ -163,9 +163,9 @@ lbm_status lbm_init_bubbles(lbm_handle *h, const lbm_bubble *bubbles, int nb, un
  * buffer and scratch planes) and rounded to FP32 there; page-locked host memory
  * makes the copy faster.  From page-locked memory, with C of 32 MB and more, at
  * least 64 rows and a stream that is not being captured, the fields go up in
- * row chunks on a second stream that the handle creates on first use (and
- * destroys with the handle), overlapped with the equilibria on the handle's
- * stream.  Synchronises the stream; returns when every copy is done. */
+ * row chunks on a second stream (created and destroyed with the handle of such
+ * a lattice), overlapped with the equilibria on the handle's stream.
+ * Synchronises the stream; returns when every copy is done. */
 lbm_status lbm_set_fields(lbm_handle *h, const double *C, const double *p, const double *ux,
                           const double *uy);
 

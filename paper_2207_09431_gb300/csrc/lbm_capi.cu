@@ -101,6 +101,24 @@ size_t lbm_required_bytes(const lbm_params *p) {
   return layout_of(*p).total;
 }
 
+// The copy stream and its events for the overlapped upload of lbm_set_fields, on handles with C of
+// 32 MB and more and chunks of at least 16 rows (the equilibria read two rows beyond their own).  A
+// copy from pageable memory returns when it is done, and 4 to 16 small copies, events and launches
+// cost more than they hide in smaller fields.  Whole and in chunks, us (GB300): C pageable 200 x 400
+// 30 and 72, 2048 x 4096 547 and 601; C, p and u pageable 200 x 400 75 and 203; C page-locked 200 x
+// 400 22 and 35, 1024 x 2048 135 and 133, 2048 x 4096 467 and 419.  Created with the handle: a
+// process's first one takes 0.2 ms, half of such an upload.
+static void create_upload_stream(lbm_handle *h) {
+  const size_t bytes = (size_t)(h->prm.ncomp - 1) * h->prm.nx * h->prm.ny * sizeof(double);
+  if (bytes < ((size_t)32 << 20) || h->prm.ny < 16 * lbm_handle::kUploadChunks) return;
+  bool ok = true;
+  for (auto &ev : h->upload_ev) ok = ok && cudaEventCreateWithFlags(&ev, cudaEventDisableTiming) == cudaSuccess;
+  if (!ok || cudaStreamCreateWithFlags(&h->copy_stream, cudaStreamNonBlocking) != cudaSuccess) {
+    h->copy_stream = nullptr;  // fields go up whole
+    cudaGetLastError();
+  }
+}
+
 lbm_status lbm_create(const lbm_params *p, void *dev_arena, size_t arena_bytes, void *cuda_stream,
                       lbm_handle **out) {
   if (!out) return LBM_E_INVAL;
@@ -146,20 +164,15 @@ lbm_status lbm_create(const lbm_params *p, void *dev_arena, size_t arena_bytes, 
     delete h;
     return LBM_E_CUDA;
   }
+  create_upload_stream(h);
   *out = h;
   return LBM_OK;
 }
 
-// Whether lbm_set_fields overlaps the upload with the initial equilibria: C of 32 MB and more in
-// page-locked memory, as the other fields, chunks of at least 16 rows (the equilibria read two rows
-// beyond their own), and a stream that is not being captured.  A copy from pageable memory returns when it
-// is done, and 4 to 16 small copies, events and launches cost more than they hide in smaller
-// fields.  Whole and in chunks, us (GB300): C pageable 200 x 400 30 and 72, 2048 x 4096 547 and 601;
-// C, p and u pageable 200 x 400 75 and 203; C page-locked 200 x 400 22 and 35, 1024 x 2048 135 and
-// 133, 2048 x 4096 467 and 419.  The copy stream and its events are created on first use.
+// Whether lbm_set_fields overlaps the upload with the initial equilibria: all fields in page-locked
+// memory, a handle that has the streams for it, and a stream that is not being captured.
 static bool upload_overlappable(lbm_handle *h, const double *C, const double *const f[3]) {
-  if (h->prm.ny < 16 * lbm_handle::kUploadChunks) return false;
-  if ((size_t)(h->prm.ncomp - 1) * h->prm.nx * h->prm.ny * sizeof(double) < ((size_t)32 << 20)) return false;
+  if (!h->copy_stream) return false;
   for (const double *p : {C, f[0], f[1], f[2]}) {
     cudaPointerAttributes a{};
     if (!p) continue;
@@ -170,17 +183,7 @@ static bool upload_overlappable(lbm_handle *h, const double *C, const double *co
     if (a.type != cudaMemoryTypeHost) return false;
   }
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-  if (cudaStreamIsCapturing(h->stream, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) return false;
-  if (!h->copy_stream && cudaStreamCreateWithFlags(&h->copy_stream, cudaStreamNonBlocking) != cudaSuccess) {
-    h->copy_stream = nullptr;
-    return false;
-  }
-  for (auto &ev : h->upload_ev)
-    if (!ev && cudaEventCreateWithFlags(&ev, cudaEventDisableTiming) != cudaSuccess) {
-      ev = nullptr;
-      return false;
-    }
-  return true;
+  return cudaStreamIsCapturing(h->stream, &cs) == cudaSuccess && cs == cudaStreamCaptureStatusNone;
 }
 
 // FP64 fields on the device, dense: C in the spare population buffer g[1] (free
