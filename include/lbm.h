@@ -184,7 +184,9 @@ lbm_status lbm_step(lbm_handle *h, long long nsteps);
 lbm_status lbm_observables(lbm_handle *h, lbm_obs *out);
 
 /* Copies field `field_id` (LBM_FIELD_*) to host_out as doubles; n is the
- * capacity of host_out in values.  Synchronises the stream. */
+ * capacity of host_out in values.  The conversion to doubles uses the spare
+ * population buffer (the one that does not hold the state) and the scratch
+ * planes, whose contents are lost.  Synchronises the stream. */
 lbm_status lbm_get_field(lbm_handle *h, int field_id, double *host_out, size_t n);
 
 /* Checkpoint: header (magic, parameters, step) then populations and tau as
@@ -209,8 +211,10 @@ const char *lbm_kernel_name(const lbm_handle *h, int i);
 lbm_status lbm_autotune(lbm_handle *h, int reps, int *chosen);
 
 /* Number of launch configurations of the step, and explicit selection of one
- * (for example a saved lbm_autotune result).  Every configuration computes the
- * same values. */
+ * (for example a saved lbm_autotune result).  A number may stand for another
+ * shape in another build of the library: a program that saves one saves the name
+ * that lbm_kernel_name gives for it as well, and looks for that name.  Every
+ * configuration computes the same values. */
 int lbm_kernel_config_count(const lbm_handle *h);
 lbm_status lbm_set_kernel_config(lbm_handle *h, int config);
 
@@ -262,7 +266,8 @@ lbm_status lbm_batch_step(lbm_batch *b, long long nsteps);
 lbm_status lbm_batch_autotune(lbm_batch *b, int reps, int *chosen);
 /* Number of launch configurations that lbm_batch_autotune chooses from in the
  * batch's current mode, and explicit selection of one (for example the one it
- * chose).  Every configuration computes the same values. */
+ * chose, in the same build of the library).  Every configuration computes the
+ * same values. */
 int lbm_batch_kernel_config_count(const lbm_batch *b);
 lbm_status lbm_batch_set_kernel_config(lbm_batch *b, int config);
 /* Persistent mode (on = 1; 0 returns to one launch per step).  lbm_batch_step

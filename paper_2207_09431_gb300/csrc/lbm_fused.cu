@@ -416,7 +416,8 @@ const char *fused_variant_name(const DevParams &P, int v) {
 // us (276 tiles), 32x8/352 6.8; then one large tile per SM, which recomputes less ring than two
 // small ones: 200 x 200 32x12/480 7.8 us (119 tiles), 32x8/352 8.8, sweep 8.1; 256 x 256
 // 32x14/544 8.7 us (152 tiles; C form 7.9), 32x8/352 8.9 (256 tiles; 8.3), sweep 10.3; 264 x 264
-// 32x8/352 8.9 us (297 tiles), sweep 10.4; 512 x 512 sweep 22.0, 32x8/352 28.3 us.
+// 32x8/352 8.9 us (297 tiles), sweep 10.4; 512 x 512 sweep 22.0, 32x8/352 28.3 us.  32x4/384/1 comes within
+// 2 % of 16x8/320 up to 128 x 128 (4.8 and 4.9 us) and is behind it above (180 x 180 8.4 and 6.0): by selection only.
 static int device_sms() {
   static const int sms = [] {
     int dev = 0, n = 0;

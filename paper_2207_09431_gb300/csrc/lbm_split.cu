@@ -251,9 +251,9 @@ __device__ __forceinline__ long long tile_node(const DevParams &P, int x, int y)
 // collision) and, with open ends, a fifth that walked the boundary rows: the
 // sources and the open ends are now part of the collision kernel.  Bound by the latency of two
 // short kernels on small lattices and by instruction issue on large ones.  Measured on a
-// GB300, one step in a replayed graph, two kernels against four (five): mixed scheme 64 x 128
-// 10.7 against 22.3 us, 200 x 400 14.2 against 29.6 us, 1024 x 2048 182 against 431 us; open
-// channel 240 x 60 11.0 against 31.2 us.  Tiles of 8 rows (fewer collisions twice, fewer CTAs)
+// GB300, us per step of lbm_step calls of 65 steps, now and with four (five) kernels: mixed scheme
+// 64 x 128 8.6 and 20.8, 200 x 400 12.4 and 28.0; open channel 240 x 60 9.3 and 28.5; mixed scheme
+// 1024 x 2048 182 and 431.  Tiles of 8 rows (fewer collisions twice, fewer CTAs)
 // ran 1 to 5 % slower above 400 x 800 at their best register budget and up to 10 % slower
 // on small lattices.  The order of a node's operations is that of the earlier kernels.
 constexpr int kTileX = 32, kTileY = 4;
@@ -396,8 +396,10 @@ __device__ __forceinline__ void collide_node(const DevParams &P, NodeCtx &n, con
 #pragma unroll
   for (int a = 0; a < 9; ++a) {
     const float G = gamma_a(a, n.ux, n.uy);
-    // (which product of the equilibrium is rounded on its own is spelled out: left to the
-    // compiler it changes with the code around it, and the results by rounding)
+    // Which product of the equilibrium is rounded on its own is spelled out: left to the
+    // compiler it changes with the code around it, and the results by rounding.  Either choice
+    // is as accurate; this one, with its split at a = 5, is what the compiler made of an earlier
+    // kernel, kept so that runs continue in the same bits.
     const float pg = phi_g(n, a, G), Gw = G - wt(a), rc = n.rho * kCs2;
     const float lin = a < 5 ? __fmaf_rn(wt(a), n.p, __fmul_rn(rc, Gw)) : __fmaf_rn(rc, Gw, __fmul_rn(wt(a), n.p));
     const float geq = lin - 0.5f * pg;
@@ -594,7 +596,8 @@ __global__ void __launch_bounds__(kCollideThreads, MINB)
 // collides the ring as well, 204 nodes for 128; here the ring costs its sources only, and the
 // stencils of a node reach two nodes instead of three.  One row's stores stay
 // together, shifted by a column in the six directions with e_x.  Bound by instruction issue.
-// Against the gather form (which this scheme took as well), us per step: 200 x 400 18.0 -> 14.2,
+// Against the gather form (which this scheme took as well), us per step, with the launches of the
+// time (200 x 400 takes 12.4 with more of them in graphs): 200 x 400 18.0 -> 14.2,
 // 1024 x 2048 225 -> 182 (157 -> 113 in this kernel), three components 256 x 256 18.3 -> 14.5.
 // Five or six CTAs per SM (fewer registers) are within 2 % of the four asked for.
 template <int NH>
@@ -753,7 +756,8 @@ __global__ void __launch_bounds__(256) k_init(DevParams P, InitFields in, float 
   n.Fs[1] = n.mu[0] * n.gC[0][1] + n.mu[1] * n.gC[1][1] + n.mu[2] * n.gC[2][1];
   n.Fb[0] = P.force_x;
   n.Fb[1] = -n.rho * P.gravity;
-  // (which product is rounded on its own is spelled out, as in k_collide_step)
+  // Which product is rounded on its own is spelled out, as in collide_node and for its reason: also the
+  // dependence on the component count, below and in the test a < NH, is an earlier compilation's.
   auto h_eq = [](float C, float G, float ph) {
     return NH == 1 ? __fmaf_rn(C, G, -0.5f * ph) : __fmaf_rn(-0.5f, ph, __fmul_rn(C, G));
   };
@@ -1116,7 +1120,8 @@ cudaError_t launch_observe(const DevParams &P, const FusedBuffers &B, int gas_co
                            cudaStream_t s) {
   const long long tiles = (long long)((P.nx + 31) / 32) * ((P.ny + 7) / 8);
   const int cap = tiles < 912 ? 228 : 456;
-  const int blocks = tiles < cap ? (int)tiles : cap;  // three CTAs per SM, fewer where each would have one tile
+  // three CTAs on each of the 152 SMs, half as many where each would have one tile or two
+  const int blocks = tiles < cap ? (int)tiles : cap;
   const int form = P.g16 ? 2 : (P.collapse_h ? 1 : 0);
   if (P.nh == 1) {
     if (form == 2) k_observe<1, 2><<<blocks, kObsThreads, 0, s>>>(P, B, gas_comp, acc, ext);
